@@ -1471,7 +1471,7 @@ __global__ void __launch_bounds__(BLOCK) k_shift(const RunDesc* __restrict__ run
 // (A, B) of a batch's runs and every segment, A's entries go into the warp's
 // on-chip table and B's entries look up theirs; the products c_A,j c_B,j and
 // G2(d)_jj c_A,j c_B,j (Eq. g2) are summed per warp.  Each warp writes its
-// own partial sums (no atomics) and k_overlap_row adds them in warp order,
+// own partial sums (no atomics) and k_overlap_row adds them in a fixed order,
 // so the result does not depend on timing.
 
 // occupation numbers of the M modes of an address (modes without a run of
@@ -1591,36 +1591,58 @@ __global__ void __launch_bounds__(128) k_overlap(const RunDesc* __restrict__ run
     if (cur_p >= 0) flush();
 }
 
-// one row of overlaps: the per-warp partial sums added in warp order; no row
-// when a run of the batch failed this step (it will be rolled back)
-static __global__ void k_overlap_row(const RunDesc* __restrict__ runs,
-                                     const OverlapDesc* __restrict__ od, unsigned nwarps) {
-    __shared__ int ok;
-    const int n = od->P * (1 + od->nq);
-    if (threadIdx.x == 0) {
-        ok = 1;
-        for (int r = 0; r < od->R; ++r)
-            if (*(volatile unsigned*)&runs[r].st->err) ok = 0;
+// Column sums of part[nwarps][n] (n <= T) by one block of T threads, in an
+// order fixed by the sizes alone: thread (group g, column c) adds rows g, g +
+// T / n, ..., then the groups are added by a tree.  Consecutive threads read
+// consecutive values and the loads of a thread do not wait for one another;
+// a thread that walked all the rows of its column alone was bound by that
+// chain of dependent adds behind strided loads (4864 rows of 15 columns: 265
+// us; this way 8 us).  Column c's sum is left in red[c].
+template <int T>
+__device__ __forceinline__ void column_sums(const double* __restrict__ part, unsigned n,
+                                            unsigned nwarps, double* red) {
+    const unsigned groups = T / n, g = threadIdx.x / n, c = threadIdx.x - g * n;
+    double s = 0.0;
+    if (g < groups) {
+#pragma unroll 8
+        for (unsigned w = g; w < nwarps; w += groups) s += part[(size_t)w * n + c];
     }
+    red[threadIdx.x] = s;
     __syncthreads();
-    if (!ok) return;
+    unsigned o = 1;
+    while (2 * o < groups) o <<= 1;
+    for (; groups > 1 && o > 0; o >>= 1) {
+        if (g < o && g + o < groups) red[threadIdx.x] += red[threadIdx.x + o * n];
+        __syncthreads();
+    }
+}
+
+// one row of overlaps: the per-warp partial sums added in a fixed order; no
+// row when a run of the batch failed this step (it will be rolled back)
+constexpr int kRowThreads = 1024;
+static __global__ void __launch_bounds__(kRowThreads)
+    k_overlap_row(const RunDesc* __restrict__ runs, const OverlapDesc* __restrict__ od,
+                  unsigned nwarps) {
+    __shared__ double red[kRowThreads];
+    const unsigned n = (unsigned)(od->P * (1 + od->nq));
+    unsigned e = 0;
+    if ((int)threadIdx.x < od->R) e = *(volatile unsigned*)&runs[threadIdx.x].st->err;
+    if (__syncthreads_or((int)e)) return;
     const unsigned long long h = *od->head;
     double* row = od->ring + (size_t)(h % od->cap) * (size_t)(1 + n);
-    for (int t = threadIdx.x; t < n; t += blockDim.x) {
-        double s = 0.0;
-        for (unsigned w = 0; w < nwarps; ++w) s += od->part[(size_t)w * n + t];
-        row[1 + t] = s;
+    column_sums<kRowThreads>(od->part, n, nwarps, red);
+    if (threadIdx.x < n) row[1 + threadIdx.x] = red[threadIdx.x];
+    if (threadIdx.x == 0) {
+        row[0] = (double)runs[0].st->step;
+        *od->head = h + 1;
     }
-    if (threadIdx.x == 0) row[0] = (double)runs[0].st->step;
-    __syncthreads();
-    if (threadIdx.x == 0) *od->head = h + 1;
 }
 
 // ---------------------------------------------------------------------------
 // excited states (Sec. 2.2): Gram-Schmidt on the step's new vectors (in
 // buffer cur ^ 1 until k_shift flips it).  For the run k being
 // orthogonalised: k_gs_dots sums c_j^T c_k and c_j^T c_j for j < k per warp,
-// k_gs_alpha adds the partials in warp order and forms alpha_j =
+// k_gs_alpha adds the partials in a fixed order and forms alpha_j =
 // (c_j^T c_k) / (c_j^T c_j), and k_gs_axpy forms c_k - sum_j alpha_j c_j
 // segment by segment in an on-chip table (subtracting j = 0, 1, ... in turn),
 // compresses every changed value by Pi with the draw of stream 0xFFFFFFFC of
@@ -1688,27 +1710,24 @@ __global__ void __launch_bounds__(128) k_gs_dots(const RunDesc* __restrict__ run
         for (unsigned i = lane; i < nl; i += 32) tk[tl[i]] = EMPTY;
         __syncwarp();
     }
-    double* part = gs->part + (size_t)gw * 2 * FQ_MAX_SPECTRAL;
+    double* part = gs->part + (size_t)gw * 2 * k;
     for (int i = 0; i < 2 * k; ++i) {
         const double v = warp_sum(acc[i]);
         if (lane == 0) part[i] = v;
     }
 }
 
-// the coefficients alpha_j of run k from the per-warp partial sums (warp
-// order); run k's norm accumulators restart for k_gs_axpy
-static __global__ void k_gs_alpha(const RunDesc* __restrict__ runs, const GsDesc* __restrict__ gs,
-                                  int k, unsigned nwarps) {
-    __shared__ double d[2 * FQ_MAX_SPECTRAL];
-    const int t = threadIdx.x;
-    if (t < 2 * k) {
-        double s = 0.0;
-        for (unsigned w = 0; w < nwarps; ++w) s += gs->part[(size_t)w * 2 * FQ_MAX_SPECTRAL + t];
-        d[t] = s;
-    }
-    __syncthreads();
-    if (t == 0) {
-        for (int j = 0; j < k; ++j) gs->alpha[j] = d[2 * j + 1] != 0.0 ? d[2 * j] / d[2 * j + 1] : 0.0;
+// the coefficients alpha_j of run k from the per-warp partial sums (added in
+// a fixed order; 102 us with one thread per sum, 4864 warps); run k's norm
+// accumulators restart for k_gs_axpy
+static __global__ void __launch_bounds__(kRowThreads)
+    k_gs_alpha(const RunDesc* __restrict__ runs, const GsDesc* __restrict__ gs, int k,
+               unsigned nwarps) {
+    __shared__ double red[kRowThreads];
+    column_sums<kRowThreads>(gs->part, 2u * (unsigned)k, nwarps, red);
+    const int j = (int)threadIdx.x;
+    if (j < k) gs->alpha[j] = red[2 * j + 1] != 0.0 ? red[2 * j] / red[2 * j + 1] : 0.0;
+    if (j == 0) {
         RunState* st = runs[k].st;
         st->norm_lo = 0;
         st->norm_hi = 0;

@@ -140,7 +140,7 @@ template <class K, int AMP, int KIND> struct Launch {
                         unsigned table, cudaStream_t s) {
         const size_t smem = (size_t)wpb * table * (sizeof(K) + sizeof(double) + sizeof(unsigned));
         k_overlap<K, AMP, KIND><<<grid, wpb * 32, smem, s>>>(d, od);
-        k_overlap_row<<<1, 256, 0, s>>>(d, od, (unsigned)(grid * wpb));
+        k_overlap_row<<<1, kRowThreads, 0, s>>>(d, od, (unsigned)(grid * wpb));
     }
     static cudaError_t prepare_overlap(size_t smem) {
         return cudaFuncSetAttribute(k_overlap<K, AMP, KIND>,
@@ -151,7 +151,7 @@ template <class K, int AMP, int KIND> struct Launch {
     static void gs(const RunDesc* d, const GsDesc* g, int k, int grid, int wpb, unsigned table,
                    cudaStream_t s) {
         k_gs_dots<K, AMP><<<grid, wpb * 32, (size_t)wpb * table * gs_dots_slot(), s>>>(d, g, k);
-        k_gs_alpha<<<1, 32, 0, s>>>(d, g, k, (unsigned)(grid * wpb));
+        k_gs_alpha<<<1, kRowThreads, 0, s>>>(d, g, k, (unsigned)(grid * wpb));
         k_gs_axpy<K, AMP, KIND><<<grid, wpb * 32, (size_t)wpb * table * gs_axpy_slot(), s>>>(d, g, k);
     }
     static cudaError_t prepare_gs(size_t smem) {
