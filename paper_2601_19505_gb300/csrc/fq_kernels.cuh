@@ -255,6 +255,9 @@ k_spawn(const RunDesc* __restrict__ runs, const unsigned* __restrict__ seg_run, 
     const ModelParams& mp = *wmp;
     unsigned g0, g1;
     warp_range(G, blockIdx.x * WPB + wib, gridDim.x * WPB, g0, g1);
+    // a warp without segments (fewer segments than warps): next_segment would
+    // take it to the first segment of the run, a second time
+    if (g0 >= g1) return;
 
     // the run of the current item: its segments [run_lo, run_hi) and per-step
     // constants
