@@ -88,9 +88,9 @@ struct fq_run {
     bool has_alloc;
     int amp, det;
     const KernelSet* ks;
-    int log2B;
     unsigned B, Cv, Cs, slots;  // slots: on-chip table slots per merge warp
     unsigned Cp;                // spawn slots per bucket in the dense primary region
+    double fill;                // steady-state spawns per bucket
     bool no_spawn_buf;          // a failed growth left no spawn buffers: the run cannot step
     RunState* st;
     StatsRow* hist;
@@ -133,6 +133,7 @@ struct fq_batch {
     cudaStream_t stream;
     RunDesc* d_desc;
     unsigned* d_seg_run;
+    unsigned* d_cuts;            // the warps' shares of the segments (batch_cuts)
     unsigned G;
     LaunchCfg cfg;
     cudaGraphExec_t g1, g16;
@@ -216,12 +217,6 @@ static unsigned next_pow2(unsigned long long x) {
     unsigned p = 1;
     while (p < x) p <<= 1;
     return p;
-}
-
-static int ilog2(unsigned x) {
-    int l = 0;
-    while ((1u << l) < x) ++l;
-    return l;
 }
 
 static int num_sms() {
@@ -531,7 +526,6 @@ static void fill_desc(const fq_run* r, RunDesc& d, unsigned seg_base) {
     d.n_ref_bkt = r->n_ref_bkt;
     d.key_x = (unsigned)r->prm.seed;
     d.key_y = (unsigned)(r->prm.seed >> 32) ^ (unsigned)(r->prm.run_id * 0x9E3779B9u);
-    d.log2B = r->log2B;
     d.B = r->B;
     d.seg_base = seg_base;
     d.Cv = r->Cv;
@@ -620,6 +614,28 @@ static void table_sizes(fq_run* r) {
         32768, next_pow2((unsigned long long)r->Cv + r->Cs));
 }
 
+// segments whose buckets fill a third of a merge warp's table of `slots`
+static double full_segments(double s_ss, unsigned slots) {
+    return std::max(1.0, std::ceil(std::min(s_ss / (slots / 3.0), 268000000.0)));
+}
+
+// Segments for s_ss spawns a step.  Large runs: full buckets, and a multiple
+// of the warps that are resident at once (16 per SM in the default launch
+// shape), so that every warp takes the same number: with a power of two, 1e6
+// walkers were 8192 buckets on 2432 warps, where some took four and most
+// three (now 7296: 8 % off the step), and 1e8 walkers 2^20 of 117 spawns
+// instead of 642048 of 171 (2 %).  Below one full bucket per warp, smaller
+// buckets on more warps, down to one round of 32 spawns: a step of 1e4
+// walkers on 12 sites took 39 us with buckets of 86 spawns and takes 33 with
+// 32, 1e5 on 20 sites 42 and 37.  Less than 64 such buckets (2000 walkers, in
+// spaces where a few addresses draw most of the spawns) stay at 100.
+static unsigned segments_for(double s_ss, unsigned slots) {
+    const double warps = num_sms() * 16.0, full = full_segments(s_ss, slots);
+    if (full > warps) return (unsigned)(std::ceil(full / warps) * warps);
+    const double fine = std::ceil(s_ss / (s_ss < 64.0 * 32.0 ? 100.0 : 32.0));
+    return (unsigned)std::max(1.0, std::min(warps, fine));
+}
+
 // per-segment capacities for totals lcap, scap over B segments (spawns
 // arrive in clumps of up to k, see fq_run_create)
 static void segment_caps(double lcap, double scap, unsigned B, double k, unsigned& Cv, unsigned& Cs) {
@@ -689,28 +705,30 @@ extern "C" int fq_run_create(fq_run** out, const fq_ham* h, const fq_params* p, 
         return FQ_ERR_INVALID;
     }
     const size_t kb = r->ks->key_bytes, ab = r->ks->amp_bytes, sb = r->ks->spawn_bytes;
-    // segments: at the expected steady state (len ~ target / threshold,
-    // spawns ~ len) the spawns into a bucket fill about a third of one merge
-    // warp's on-chip table (the table holds spawned addresses only)
+    // segments for the expected steady state (len ~ target / threshold, spawns
+    // ~ len); the merge's table holds a bucket's spawned addresses only
     r->slots = warp_slots(r->ks);
     double l_ss = std::min(p->target / th, dim), s_ss = 1.1 * p->target / th;
     if (r->det) {
         l_ss = std::min(lcap, dim);
         s_ss = l_ss * (double)max_offdiag(h->mp);
     }
-    const unsigned long long want =
-        (unsigned long long)std::ceil(s_ss / (r->slots / 3.0));
-    r->B = next_pow2(std::max<unsigned long long>(1, std::min<unsigned long long>(want, 1ull << 28)));
+    r->B = segments_for(s_ss, r->slots);
     {
         // spawns arrive in clumps (one address receives spawns from many
         // sources; every neighbour's in the deterministic limit), so the
         // bucket count fluctuates like a compound Poisson sum with clump size k
         const double k = r->det ? (double)max_offdiag(h->mp) : 8.0;
+        unsigned c = 0;
         segment_caps(lcap, scap, r->B, k, r->Cv, r->Cs);
+        // spawns come in clumps of one address, which a small bucket feels
+        // more: it has the room of a full one
+        segment_caps(lcap, scap, (unsigned)std::min<double>(r->B, full_segments(s_ss, r->slots)), k,
+                     c, r->Cs);
         r->Cp = primary_slots(s_ss, r->B, k, r->Cs);
+        r->fill = std::min(s_ss / r->B, 1e6);
         table_sizes(r);
     }
-    r->log2B = ilog2(r->B);
     const unsigned B = r->B;
 
     bool ok = true;
@@ -945,7 +963,7 @@ extern "C" int fq_run_set_reference(fq_run* r, const fq_key* keys, const double*
     CK(bufs.get(&d_tv, sizeof(double) * T));
     CK(bufs.get(&d_tseg, sizeof(unsigned) * T));
     CK(cudaMemcpy(d_off, off.data(), sizeof(unsigned) * (n + 1), cudaMemcpyHostToDevice));
-    r->ks->ref_terms(mp, d_refs, d_y, (int)n, d_off, d_tk, d_th, d_tv, d_tseg, r->log2B, 0);
+    r->ks->ref_terms(mp, d_refs, d_y, (int)n, d_off, d_tk, d_th, d_tv, d_tseg, r->B, 0);
     CK(cudaDeviceSynchronize());
     std::vector<unsigned char> tk(kb * T);
     std::vector<double> th(T), tv(T);
@@ -1061,6 +1079,8 @@ static void batch_release(fq_batch* b) {
     if (b->g16) cudaGraphExecDestroy(b->g16);
     if (b->d_desc) cudaFree(b->d_desc);
     if (b->d_seg_run) cudaFree(b->d_seg_run);
+    if (b->d_cuts) cudaFree(b->d_cuts);
+    b->d_cuts = nullptr;
     b->g1 = b->g16 = nullptr;
     b->d_desc = nullptr;
     b->d_seg_run = nullptr;
@@ -1242,6 +1262,64 @@ static std::vector<LaunchCfg> batch_shapes(fq_batch* b, unsigned slots) {
     return v;
 }
 
+// Every launch shape's shares of the batch's segments: cuts[w] is warp w's
+// first segment.  A share lies within one run, and no share's expected work is
+// more than the smallest bound for which the warps suffice.  A bucket costs
+// about as much as 32 spawns before its first one (batch of 64 runs with
+// buckets of 32 to 170 spawns: 42.9 ms a chunk with 24, 42.4 with 48, 47.7
+// with 8, 45.6 with 96).
+static std::vector<unsigned> share_cuts(const fq_batch* b, unsigned nw) {
+    const std::vector<fq_run*>& runs = b->runs;
+    auto parts = [](const fq_run* r, double most) {  // shares of run r: at most `most` each
+        const double per = std::max(1.0, std::floor(most / (32.0 + r->fill)));  // segments
+        return (unsigned)std::ceil(r->B / per);
+    };
+    double lo = 0.0, hi = 0.0;
+    for (const fq_run* r : runs) hi = std::max(hi, r->B * (32.0 + r->fill));
+    for (int i = 0; i < 40; ++i) {
+        const double mid = 0.5 * (lo + hi);
+        unsigned long long n = 0;
+        for (const fq_run* r : runs) n += parts(r, mid);
+        (n <= nw ? hi : lo) = mid;
+    }
+    std::vector<unsigned> cuts;
+    unsigned base = 0;
+    for (const fq_run* r : runs) {
+        const unsigned k = parts(r, hi);
+        for (unsigned i = 0; i < k; ++i)
+            cuts.push_back(base + (unsigned)((unsigned long long)r->B * i / k));
+        base += r->B;
+    }
+    cuts.resize(nw + 1, base);  // warps beyond the shares have none
+    return cuts;
+}
+
+static int batch_cuts(fq_batch* b) {
+    if (b->runs.size() < 2) return FQ_OK;
+    std::vector<unsigned> all;
+    std::vector<std::pair<unsigned, size_t>> have;  // warps, offset of their cuts
+    auto of = [&](int warps) {
+        for (const auto& h : have)
+            if (h.first == (unsigned)warps) return h.second;
+        const std::vector<unsigned> c = share_cuts(b, (unsigned)warps);
+        have.push_back({(unsigned)warps, all.size()});
+        all.insert(all.end(), c.begin(), c.end());
+        return have.back().second;
+    };
+    std::vector<size_t> so, mo;
+    for (const LaunchCfg& c : b->shapes) {
+        so.push_back(of(c.spawn_grid * c.spawn_wpb));
+        mo.push_back(of(c.merge_grid * c.merge_wpb));
+    }
+    CK(cudaMalloc((void**)&b->d_cuts, sizeof(unsigned) * all.size()));
+    CK(cudaMemcpy(b->d_cuts, all.data(), sizeof(unsigned) * all.size(), cudaMemcpyHostToDevice));
+    for (size_t i = 0; i < b->shapes.size(); ++i) {
+        b->shapes[i].spawn_cuts = b->d_cuts + so[i];
+        b->shapes[i].merge_cuts = b->d_cuts + mo[i];
+    }
+    return FQ_OK;
+}
+
 static int batch_build(fq_batch* b) {
     const size_t nr = b->runs.size();
     b->gens.resize(nr);
@@ -1265,6 +1343,10 @@ static int batch_build(fq_batch* b) {
     CK(cudaMemcpy(b->d_seg_run, seg_run.data(), sizeof(unsigned) * base, cudaMemcpyHostToDevice));
     CK(b->ks->prepare(200u * 1024u));
     b->shapes = batch_shapes(b, slots);
+    for (LaunchCfg& c : b->shapes) {  // every run has a warp of its own
+        c.spawn_grid = std::max(c.spawn_grid, ((int)nr + c.spawn_wpb - 1) / c.spawn_wpb);
+        c.merge_grid = std::max(c.merge_grid, ((int)nr + c.merge_wpb - 1) / c.merge_wpb);
+    }
     // scratch tables for the largest number of merge warps of any shape
     size_t warps = 0;
     for (const LaunchCfg& c : b->shapes) warps = std::max(warps, (size_t)c.merge_grid * c.merge_wpb);
@@ -1318,7 +1400,8 @@ static int batch_build(fq_batch* b) {
         c.sort_elems = se;
     }
     {
-        int rc = overlaps_build(b);
+        int rc = batch_cuts(b);
+        if (!rc) rc = overlaps_build(b);
         if (!rc) rc = gs_build(b);
         if (rc) return rc;
     }
@@ -1345,6 +1428,7 @@ static int batch_new(fq_run* const* runs, int n, bool owned, fq_batch** out) {
     b->owned_by_run = owned;
     b->d_desc = nullptr;
     b->d_seg_run = nullptr;
+    b->d_cuts = nullptr;
     b->g1 = b->g16 = nullptr;
     b->scratch = nullptr;
     b->scratch_bytes = 0;
@@ -1781,6 +1865,7 @@ static int autotune(fq_batch* b, int steps) {
         c.spawn_var = s2.spawn_var;
         c.spawn_wpb = s2.spawn_wpb;
         c.spawn_grid = s2.spawn_grid;
+        c.spawn_cuts = s2.spawn_cuts;
         return c;
     };
     if (e == cudaSuccess) enqueue_steps(b, 1, b->stream);  // warm
@@ -1826,6 +1911,7 @@ static int autotune(fq_batch* b, int steps) {
     best.spawn_var = sc[bs].spawn_var;
     best.spawn_wpb = sc[bs].spawn_wpb;
     best.spawn_grid = sc[bs].spawn_grid;
+    best.spawn_cuts = sc[bs].spawn_cuts;
     b->cfg = best;
     if (b->g1) cudaGraphExecDestroy(b->g1);
     if (b->g16) cudaGraphExecDestroy(b->g16);

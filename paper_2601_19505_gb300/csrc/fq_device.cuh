@@ -195,7 +195,8 @@ __device__ __forceinline__ unsigned pick(uint4 w, unsigned m) {
     return (unsigned)(((unsigned long long)w.z * (unsigned long long)m) >> 32);
 }
 
-// segment hash; the segment is the top bits.  64-bit addresses: one
+// segment hash; the segment is its high word scaled to the number of segments
+// (segment_of).  64-bit addresses: one
 // multiply by an odd constant (multiplicative hashing), unrelated to the
 // golden-ratio constant of the merge table's slot hash (with related
 // constants, small addresses that share a segment would also share a few
@@ -206,8 +207,10 @@ __device__ __forceinline__ uint64_t seg_hash(uint64_t k) { return k * 0xD6E8FEB8
 __device__ __forceinline__ uint64_t seg_hash(u128 k) {
     return ((uint64_t)k ^ ((uint64_t)(k >> 64) * 0xC2B2AE3D27D4EB4Full)) * 0xD6E8FEB86659FD93ull;
 }
-__device__ __forceinline__ unsigned segment_of(uint64_t mixed, int log2B) {
-    return log2B ? (unsigned)(mixed >> (64 - log2B)) : 0u;
+// the segment of a hash among B of them, any B: floor(hash B / 2^32) of the
+// hash's high word (one multiply; a shift by log2 B would tie B to powers of 2)
+__device__ __forceinline__ unsigned segment_of(uint64_t mixed, unsigned B) {
+    return __umulhi((unsigned)(mixed >> 32), B);
 }
 
 // ---------------------------------------------------------------------------

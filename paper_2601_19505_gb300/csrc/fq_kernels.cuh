@@ -18,7 +18,7 @@
 //
 // Layout: the vector of a run is hash-segmented (the paper's PDVec segments,
 // Sec. 6.4, as thousands of small segments sized for one merge warp's
-// on-chip table): segment b = top log2(B) bits of seg_hash(address), capacity Cv
+// on-chip table): segment b = segment_of(seg_hash(address), B), capacity Cv
 // entries each, structure-of-arrays keys/amplitudes.  Spawn buckets use the
 // same segment map with capacity Cs.  All sizes and pointers are read from
 // device memory, so one captured CUDA graph replays any number of steps.
@@ -163,6 +163,21 @@ __device__ __forceinline__ void warp_range(unsigned G, unsigned w, unsigned nw, 
     g0 = (unsigned)(((unsigned long long)G * w) / nw);
     g1 = (unsigned)(((unsigned long long)G * (w + 1)) / nw);
 }
+// ... or between the host's cuts: in a batch of runs whose segments hold
+// unequal work, shares of equal work, each of segments of one run (batch_cuts
+// in fq_api.cu).  With equal counts of segments, a warp among the runs of full
+// buckets had up to five times the work of one among the runs of small ones,
+// and a batch of 64 runs of 1e4 to 1e6 walkers took 1.92 ms a step instead of
+// 1.33.
+__device__ __forceinline__ void warp_range(const unsigned* __restrict__ cuts, unsigned G, unsigned w,
+                                           unsigned nw, unsigned& g0, unsigned& g1) {
+    if (cuts) {
+        g0 = cuts[w];
+        g1 = cuts[w + 1];
+    } else {
+        warp_range(G, w, nw, g0, g1);
+    }
+}
 
 // ---------------------------------------------------------------------------
 // asynchronous global -> shared copies (cp.async, 16-byte chunks; a chunk
@@ -230,7 +245,8 @@ template <class K, int AMP, int CH, int KIND> struct SpawnSmem {
 
 template <class K, int AMP, int KIND, int V, int IPT>
 __global__ void __launch_bounds__(Var<V>::WPB * 32, Var<V>::MINB)
-k_spawn(const RunDesc* __restrict__ runs, const unsigned* __restrict__ seg_run, unsigned G) {
+k_spawn(const RunDesc* __restrict__ runs, const unsigned* __restrict__ seg_run, unsigned G,
+        const unsigned* __restrict__ cuts) {
     constexpr int WPB = Var<V>::WPB;
     typedef typename AmpT<AMP>::A A;
     typedef typename AmpT<AMP>::S S;
@@ -247,38 +263,49 @@ k_spawn(const RunDesc* __restrict__ runs, const unsigned* __restrict__ seg_run, 
     CO* const wcoef = (CO*)(wbase + SM::coef_off);
     unsigned* const woff = (unsigned*)(wbase + SM::off_off);
     unsigned* const wm = (unsigned*)(wbase + SM::m_off);
-    // the current run's model parameters, copied into the warp's shared
-    // memory when the run is entered: read there, they are not reloaded
+    // the run's model parameters, copied into the warp's shared memory: read
+    // there, they are not reloaded
     // through L1 after every spawn store (which the compiler cannot tell
     // apart from the run descriptor)
     ModelParams* const wmp = (ModelParams*)(wbase + SM::mp_off);
     const ModelParams& mp = *wmp;
     unsigned g0, g1;
-    warp_range(G, blockIdx.x * WPB + wib, gridDim.x * WPB, g0, g1);
-    // a warp without segments (fewer segments than warps): next_segment would
-    // take it to the first segment of the run, a second time
-    if (g0 >= g1) return;
+    warp_range(cuts, G, blockIdx.x * WPB + wib, gridDim.x * WPB, g0, g1);
+    if (g0 >= g1) return;  // fewer segments than warps
 
-    // the run of the current item: its segments [run_lo, run_hi) and per-step
-    // constants
-    const RunDesc* R = nullptr;
-    unsigned run_lo = 0, run_hi = 0;
-    unsigned err = 0;
-    const K* vk0 = nullptr;
-    const A* va0 = nullptr;
-    const unsigned* vcnt = nullptr;
-    unsigned Cv = 0, Cs = 0, Cp = 0, stepno = 0;
-    void* sk = nullptr;
-    void* sv = nullptr;
-    unsigned* sfill = nullptr;
-    int log2B = 0;
-    double dt = 0.0;
-    uint2 rkey = make_uint2(0, 0);
-    int early = 0;
+    // the range's run (a range never crosses runs): its first segment and
+    // per-step constants
+    const RunDesc* const R = runs + seg_run[g0];
+    // lane 0 reads, the warp shares: another warp may set an error bit
+    unsigned err = 0, cur = 0;
+    if (lane == 0) {
+        err = *(volatile unsigned*)&R->st->err;
+        cur = (unsigned)R->st->cur;
+    }
+    err = __shfl_sync(0xFFFFFFFFu, err, 0);
+    cur = __shfl_sync(0xFFFFFFFFu, cur, 0);
+    if (err) return;
+    const unsigned run_lo = R->seg_base, nB = R->B;
+    const K* const vk0 = (const K*)R->vkeys[cur];
+    const A* const va0 = (const A*)R->vamps[cur];
+    const unsigned* const vcnt = R->vcount[cur];
+    const unsigned Cv = R->Cv, Cs = R->Cs, Cp = R->Cp;
+    void* const sk = R->skeys;
+    void* const sv = R->samps;
+    unsigned* const sfill = R->sfill;
+    const double dt = R->st->dt;
+    const unsigned stepno = (unsigned)(R->st->step + 1);
+    const uint2 rkey = make_uint2(R->key_x, R->key_y);
+    const int early = R->early;
     // per-source constants of the run, in registers for the same reason
-    int r_det = 0, r_trel_one = 0, r_mmax = 0;
-    double r_trel = 0.0;
+    const int r_det = R->mode_det, r_trel_one = R->trel_one, r_mmax = R->mmax;
+    const double r_trel = R->t_rel;
     const typename AmpT<AMP>::C* r_coef = nullptr;
+    if constexpr (AMP == FQ_AMP_F32) r_coef = R->coef32;
+    else if constexpr (AMP == FQ_AMP_F64) r_coef = R->coef64;
+    for (unsigned i = (unsigned)lane; i < (unsigned)(SM::mp_bytes / 4); i += 32u)
+        ((unsigned*)wmp)[i] = ((const unsigned*)&R->mp)[i];
+    __syncwarp();
     unsigned n_ex = 0, n_inex = 0, n_sp = 0;
 
     // the spawn whose bucket slot is being reserved (stored one spawn later)
@@ -290,77 +317,21 @@ k_spawn(const RunDesc* __restrict__ runs, const unsigned* __restrict__ seg_run, 
     auto flush_pending = [&]() {
         if (!ph) return;
         if (pp < Cs) {
-            SpawnIO<K, S>::store(sk, sv, spawn_slot(pb, pp, Cp, Cs, run_hi - run_lo), pd, pv);
+            SpawnIO<K, S>::store(sk, sv, spawn_slot(pb, pp, Cp, Cs, nB), pd, pv);
         } else {
             atomicOr(&R->st->err, FQ_DERR_SPAWN_CAP);
         }
         ph = false;
     };
-    auto flush_counts = [&]() {
-        const unsigned long long a = warp_sum((unsigned long long)n_ex);
-        const unsigned long long i = warp_sum((unsigned long long)n_inex);
-        const unsigned long long p = warp_sum((unsigned long long)n_sp);
-        if (lane == 0) {
-            if (a) atomicAdd(&R->st->n_exact, a);
-            if (i) atomicAdd(&R->st->n_inexact, i);
-            if (p) atomicAdd(&R->st->n_spawns, p);
-        }
-        n_ex = n_inex = n_sp = 0;
-    };
-    // make run r current (warp-uniform)
-    auto enter_run = [&](int r) {
-        if (R) {
-            flush_pending();
-            flush_counts();
-        }
-        R = runs + r;
-        // lane 0 reads, the warp shares: another warp may set an error bit
-        unsigned e = 0, c = 0;
-        if (lane == 0) {
-            e = *(volatile unsigned*)&R->st->err;
-            c = (unsigned)R->st->cur;
-        }
-        err = __shfl_sync(0xFFFFFFFFu, e, 0);
-        const unsigned cur = __shfl_sync(0xFFFFFFFFu, c, 0);
-        run_lo = R->seg_base;
-        run_hi = run_lo + R->B;
-        vk0 = (const K*)R->vkeys[cur];
-        va0 = (const A*)R->vamps[cur];
-        vcnt = R->vcount[cur];
-        Cv = R->Cv;
-        Cs = R->Cs;
-        Cp = R->Cp;
-        sk = R->skeys;
-        sv = R->samps;
-        sfill = R->sfill;
-        log2B = R->log2B;
-        dt = R->st->dt;
-        stepno = (unsigned)(R->st->step + 1);
-        rkey = make_uint2(R->key_x, R->key_y);
-        early = R->early;
-        r_det = R->mode_det;
-        r_trel_one = R->trel_one;
-        r_trel = R->t_rel;
-        r_mmax = R->mmax;
-        if constexpr (AMP == FQ_AMP_F32) r_coef = R->coef32;
-        else if constexpr (AMP == FQ_AMP_F64) r_coef = R->coef64;
-        __syncwarp();  // every lane is done with the previous run's parameters
-        for (unsigned i = (unsigned)lane; i < (unsigned)(SM::mp_bytes / 4); i += 32u)
-            ((unsigned*)wmp)[i] = ((const unsigned*)&R->mp)[i];
-        __syncwarp();
-    };
-    // the next non-empty segment of the current run at or after g; the end
-    // of the run's part of the range if none (n = its entry count)
+    // the next non-empty segment at or after g; g1 if none (n = its entry count)
     // the count of segment pre_g, loaded one segment ahead of its use
     unsigned pre_g = 0xFFFFFFFFu, pre_n = 0;
     auto next_segment = [&](unsigned g, unsigned& n) -> unsigned {
-        const unsigned hi = min(g1, run_hi);
-        if (err) return hi;
-        for (; g < hi; ++g) {
+        for (; g < g1; ++g) {
             n = g == pre_g ? pre_n : vcnt[g - run_lo];
             if (n) return g;
         }
-        return hi;
+        return g1;
     };
     auto stage = [&](unsigned g, unsigned c0, unsigned cn, int b) {
         const size_t e0 = (size_t)(g - run_lo) * Cv + c0;
@@ -416,7 +387,7 @@ k_spawn(const RunDesc* __restrict__ runs, const unsigned* __restrict__ seg_run, 
     auto emit = [&](bool has, K dest, S val) {
         unsigned bk = 0, pos = 0;
         if (has) {
-            bk = segment_of(seg_hash(dest), log2B);
+            bk = segment_of(seg_hash(dest), nB);
             pos = atomicAdd(&sfill[bk], 1u);
             ++n_sp;
         }
@@ -431,35 +402,26 @@ k_spawn(const RunDesc* __restrict__ runs, const unsigned* __restrict__ seg_run, 
     };
 
     // current item (segment g, entries [c0, c0 + CH) of n), staged in buffer b
-    unsigned g = g0, c0 = 0, n = 0;
+    unsigned c0 = 0, n = 0;
+    unsigned g = next_segment(g0, n);
     int b = 0;
-    bool staged = false;
-    while (true) {
-        if (g < g1 && (g < run_lo || g >= run_hi)) {
-            enter_run((int)seg_run[g]);
-            staged = false;
-        }
-        if (!staged) {
-            g = next_segment(g, n);
-            if (g >= g1) break;
-            if (g >= run_hi) continue;
-            c0 = 0;
-            stage(g, 0, min((unsigned)CH, n), b);
-        }
+    if (g < g1) stage(g, 0, min((unsigned)CH, n), b);
+    while (g < g1) {
         const unsigned cn = min((unsigned)CH, n - c0);
         cp_async_wait_all();
         __syncwarp();
-        // stage the next item of the same run into the other buffer
+        // stage the next item into the other buffer
         unsigned ng = g, nc0 = c0 + CH, nn = n;
         if (nc0 >= n) {
             nc0 = 0;
             ng = next_segment(g + 1, nn);
         }
-        staged = ng < g1 && ng < run_hi;
-        if (staged) stage(ng, nc0, min((unsigned)CH, nn - nc0), b ^ 1);
-        if (staged && ng + 1 < min(g1, run_hi) && pre_g != ng + 1) {
-            pre_g = ng + 1;
-            pre_n = vcnt[pre_g - run_lo];
+        if (ng < g1) {
+            stage(ng, nc0, min((unsigned)CH, nn - nc0), b ^ 1);
+            if (ng + 1 < g1 && pre_g != ng + 1) {
+                pre_g = ng + 1;
+                pre_n = vcnt[pre_g - run_lo];
+            }
         }
 
         const K* wkey = in_key + b * CH;
@@ -544,14 +506,18 @@ k_spawn(const RunDesc* __restrict__ runs, const unsigned* __restrict__ seg_run, 
         }
         __syncwarp();  // every lane is done with buffer b
         g = ng;
-        if (!staged) continue;
         c0 = nc0;
         n = nn;
         b ^= 1;
     }
-    if (R) {
-        flush_pending();
-        flush_counts();
+    flush_pending();
+    const unsigned long long ex = warp_sum((unsigned long long)n_ex);
+    const unsigned long long inex = warp_sum((unsigned long long)n_inex);
+    const unsigned long long nsp = warp_sum((unsigned long long)n_sp);
+    if (lane == 0) {
+        if (ex) atomicAdd(&R->st->n_exact, ex);
+        if (inex) atomicAdd(&R->st->n_inexact, inex);
+        if (nsp) atomicAdd(&R->st->n_spawns, nsp);
     }
 }
 
@@ -683,11 +649,14 @@ __device__ __forceinline__ bool compress(typename AmpT<AMP>::ACC w, const StepCo
 
 // per-warp totals of one run, carried across buckets
 struct MergeAcc {
-    unsigned long long nlo, nhi, nlen;
+    unsigned long long nlo, nhi;   // exact norm terms
     double nfp;
+    unsigned nlen, ntheta;         // stored values of this lane; those of magnitude theta
     bool full, over, range_bad;
-    unsigned long long ntheta;  // stored values of magnitude theta (a power of two)
     unsigned n_onchip, n_scratch;  // buckets summed in each kind of table (warp-uniform)
+    __device__ __forceinline__ MergeAcc()
+        : nlo(0), nhi(0), nfp(0.0), nlen(0), ntheta(0), full(false), over(false),
+          range_bad(false), n_onchip(0), n_scratch(0) {}
 };
 
 // the two halves of Pi for one value, for early compression (Sec. 7.1, Eq.
@@ -727,9 +696,10 @@ __device__ __forceinline__ bool pi_below(V& v, uint4 r, const RunDesc* R) {
 // add a warp's share of one run's step totals to the run's accumulators
 __device__ __forceinline__ void merge_flush(const RunDesc* R, MergeAcc a, int lane) {
     unsigned long long nlo = a.nlo, nhi = a.nhi;
-    add128(nlo, nhi, a.ntheta << 52, a.ntheta >> 12);  // the values of magnitude theta
+    const unsigned long long nt = a.ntheta;
+    add128(nlo, nhi, nt << 52, nt >> 12);  // the values of magnitude theta
     warp_sum128(nlo, nhi);
-    const unsigned long long nlen = warp_sum(a.nlen);
+    const unsigned long long nlen = warp_sum((unsigned long long)a.nlen);
     const double nfp = warp_sum(a.nfp);
     const bool f = __any_sync(0xFFFFFFFFu, a.full), o = __any_sync(0xFFFFFFFFu, a.over),
                b = __any_sync(0xFFFFFFFFu, a.range_bad);
@@ -1191,7 +1161,8 @@ template <class K, int AMP, int ANN> __host__ __device__ constexpr size_t merge_
 template <class K, int AMP, int KIND, int V, int ANN>
 __global__ void __launch_bounds__(Var<V>::WPB * 32, Var<V>::MINB)
 k_merge(const RunDesc* __restrict__ runs, const unsigned* __restrict__ seg_run, unsigned G,
-        unsigned SW, unsigned char* __restrict__ scratch, unsigned SS) {
+        unsigned SW, unsigned char* __restrict__ scratch, unsigned SS,
+        const unsigned* __restrict__ cuts) {
     constexpr int WPB = Var<V>::WPB;
     typedef typename AmpT<AMP>::ACC ACC;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1220,35 +1191,29 @@ k_merge(const RunDesc* __restrict__ runs, const unsigned* __restrict__ seg_run, 
     }
     __syncwarp();
     unsigned g0, g1;
-    warp_range(G, gw, gridDim.x * WPB, g0, g1);
+    warp_range(cuts, G, gw, gridDim.x * WPB, g0, g1);
 
-    const RunDesc* R = nullptr;
-    unsigned run_lo = 0, run_hi = 0;  // segments of the current run
+    if (g0 >= g1) return;
+    // The range's run: a range never crosses runs.  (A loop over the runs of a
+    // range, with totals flushed and restarted between them, counted wrongly
+    // for integer walkers: a batch's second run in a warp started from stale
+    // registers, while the same source steps right on a CPU.)
+    const RunDesc* const R = runs + seg_run[g0];
+    // lane 0 reads, the warp shares: another warp may set an error bit
     unsigned err = 0, cur = 0;
-    MergeAcc acc = {0, 0, 0, 0.0, false, false, false, 0, 0, 0};
+    if (lane == 0) {
+        err = *(volatile unsigned*)&R->st->err;
+        cur = (unsigned)R->st->cur;
+    }
+    err = __shfl_sync(0xFFFFFFFFu, err, 0);
+    cur = __shfl_sync(0xFFFFFFFFu, cur, 0);
+    if (err) return;
+    MergeAcc acc;
     // counts of buckets ahead_g and ahead2_g, loaded before they are needed
     unsigned ahead_g = 0xFFFFFFFFu, ahead2_g = 0xFFFFFFFFu;
     unsigned a1_old = 0, a1_sp = 0, a2_old = 0, a2_sp = 0;
 
     for (unsigned g = g0; g < g1; ++g) {
-        if (g < run_lo || g >= run_hi) {  // warp-uniform
-            if (R) {
-                merge_flush(R, acc, lane);
-                acc = MergeAcc{0, 0, 0, 0.0, false, false, false, 0, 0, 0};
-            }
-            R = runs + seg_run[g];
-            run_lo = R->seg_base;
-            run_hi = run_lo + R->B;
-            // lane 0 reads, the warp shares: another warp may set an error bit
-            unsigned e = 0, c = 0;
-            if (lane == 0) {
-                e = *(volatile unsigned*)&R->st->err;
-                c = (unsigned)R->st->cur;
-            }
-            err = __shfl_sync(0xFFFFFFFFu, e, 0);
-            cur = __shfl_sync(0xFFFFFFFFu, c, 0);
-        }
-        if (err) continue;
         const unsigned seg = g - R->seg_base;
         // this bucket's counts (loaded one bucket ahead when it was the next);
         // then the next bucket's data is prefetched into L2 and the counts of
@@ -1261,8 +1226,7 @@ k_merge(const RunDesc* __restrict__ runs, const unsigned* __restrict__ seg_run, 
             n_old = R->vcount[cur][seg];
             n_sp = R->sfill[seg];
         }
-        const unsigned g_end = min(g1, R->seg_base + R->B);
-        if (g + 1 < g_end) {
+        if (g + 1 < g1) {
             unsigned o1, s1;
             if (g + 1 == ahead2_g) {
                 o1 = a2_old;
@@ -1305,7 +1269,7 @@ k_merge(const RunDesc* __restrict__ runs, const unsigned* __restrict__ seg_run, 
             ahead_g = g + 1;
             a1_old = o1;
             a1_sp = s1;
-            if (g + 2 < g_end) {
+            if (g + 2 < g1) {
                 ahead2_g = g + 2;
                 a2_old = R->vcount[cur][seg + 2];
                 a2_sp = R->sfill[seg + 2];
@@ -1339,7 +1303,7 @@ k_merge(const RunDesc* __restrict__ runs, const unsigned* __restrict__ seg_run, 
             acc.full = true;  // even the scratch table cannot hold this bucket
         }
     }
-    if (R) merge_flush(R, acc, lane);
+    merge_flush(R, acc, lane);
 }
 
 // scratch tables start empty (keys EMPTY, sums 0); each use leaves them so
@@ -1772,7 +1736,7 @@ __global__ void __launch_bounds__(128) k_gs_axpy(const RunDesc* __restrict__ run
     const int nq = R->norm_q, det = R->mode_det;
     double alpha[FQ_MAX_SPECTRAL];
     for (int j = 0; j < k; ++j) alpha[j] = gs->alpha[j];
-    MergeAcc acc = {0, 0, 0, 0.0, false, false, false, 0, 0, 0};
+    MergeAcc acc;
     unsigned g0, g1;
     warp_range(gs->B, gw, nw, g0, g1);
     for (unsigned seg = g0; seg < g1; ++seg) {
@@ -1872,7 +1836,7 @@ __global__ void k_seed(const RunDesc* __restrict__ R, const K* __restrict__ keys
     if (i >= n) return;
     const int cur = R->st->cur;
     const K key = keys[i];
-    const unsigned b = segment_of(seg_hash(key), R->log2B);
+    const unsigned b = segment_of(seg_hash(key), R->B);
     const unsigned pos = atomicAdd(&R->vcount[cur][b], 1u);
     if (pos < R->Cv) {
         ((K*)R->vkeys[cur])[(size_t)b * R->Cv + pos] = key;
@@ -1906,7 +1870,7 @@ __global__ void k_lookup(const RunDesc* __restrict__ R, const K* __restrict__ q,
     if (i >= n) return;
     const int cur = R->st->cur;
     const K key = q[i];
-    const unsigned b = segment_of(seg_hash(key), R->log2B);
+    const unsigned b = segment_of(seg_hash(key), R->B);
     const unsigned c = min(R->vcount[cur][b], R->Cv);
     const K* vk = (const K*)R->vkeys[cur] + (size_t)b * R->Cv;
     const A* va = (const A*)R->vamps[cur] + (size_t)b * R->Cv;
@@ -1971,7 +1935,7 @@ __global__ void k_column(ModelParams mp, K key, K* dest, double* val, unsigned c
 template <class K, int KIND>
 __global__ void k_ref_terms(ModelParams mp, const K* __restrict__ refs, const double* __restrict__ y,
                             int n, const unsigned* __restrict__ off, K* tkeys, double* th,
-                            double* tv, unsigned* tseg, int log2B) {
+                            double* tv, unsigned* tseg, unsigned B) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
     typedef Model<KIND> MD;
@@ -1982,7 +1946,7 @@ __global__ void k_ref_terms(ModelParams mp, const K* __restrict__ refs, const do
     tkeys[o] = key;
     th[o] = y[r] * MD::diagonal(mp, key);
     tv[o] = y[r];
-    tseg[o] = segment_of(seg_hash(key), log2B);
+    tseg[o] = segment_of(seg_hash(key), B);
     ++o;
     for (unsigned k = 0; k < m; ++k, ++o) {
         double hv;
@@ -1990,7 +1954,7 @@ __global__ void k_ref_terms(ModelParams mp, const K* __restrict__ refs, const do
         tkeys[o] = d;
         th[o] = y[r] * hv;
         tv[o] = 0.0;
-        tseg[o] = segment_of(seg_hash(d), log2B);
+        tseg[o] = segment_of(seg_hash(d), B);
     }
 }
 

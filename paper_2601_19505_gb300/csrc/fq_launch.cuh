@@ -18,7 +18,8 @@ template <class K, int AMP, int KIND> struct Launch {
     template <int V> static void spawn_v(const LaunchCfg& c, const RunDesc* d, const unsigned* sr,
                                          unsigned G, cudaStream_t s) {
         constexpr int W = Var<V>::WPB;
-        k_spawn<K, AMP, KIND, V, 4><<<c.spawn_grid, W * 32, spawn_smem(W), s>>>(d, sr, G);
+        k_spawn<K, AMP, KIND, V, 4><<<c.spawn_grid, W * 32, spawn_smem(W), s>>>(d, sr, G,
+                                                                                  c.spawn_cuts);
     }
     static void spawn(const LaunchCfg& c, const RunDesc* d, const unsigned* sr, unsigned G,
                       cudaStream_t s) {
@@ -32,11 +33,11 @@ template <class K, int AMP, int KIND> struct Launch {
         if (c.ann == FQ_ANN_SORT_ARM) {
             const size_t smem = (size_t)W * merge_warp_bytes<K, AMP, FQ_ANN_SORT_ARM>(c.slots);
             k_merge<K, AMP, KIND, V, FQ_ANN_SORT_ARM><<<c.merge_grid, W * 32, smem, s>>>(
-                d, sr, G, c.slots, c.sort_scratch, c.sort_elems);
+                d, sr, G, c.slots, c.sort_scratch, c.sort_elems, c.merge_cuts);
         } else {
             const size_t smem = (size_t)W * merge_warp_bytes<K, AMP, FQ_ANN_HASH_ARM>(c.slots);
             k_merge<K, AMP, KIND, V, FQ_ANN_HASH_ARM><<<c.merge_grid, W * 32, smem, s>>>(
-                d, sr, G, c.slots, c.scratch, c.scratch_slots);
+                d, sr, G, c.slots, c.scratch, c.scratch_slots, c.merge_cuts);
         }
     }
     static void merge(const LaunchCfg& c, const RunDesc* d, const unsigned* sr, unsigned G,
@@ -132,9 +133,9 @@ template <class K, int AMP, int KIND> struct Launch {
     }
     static void ref_terms(const ModelParams& mp, const void* refs, const double* y, int n,
                           const unsigned* off, void* tkeys, double* th, double* tv,
-                          unsigned* tseg, int log2B, cudaStream_t s) {
+                          unsigned* tseg, unsigned B, cudaStream_t s) {
         k_ref_terms<K, KIND><<<(n + 63) / 64, 64, 0, s>>>(mp, (const K*)refs, y, n, off,
-                                                          (K*)tkeys, th, tv, tseg, log2B);
+                                                          (K*)tkeys, th, tv, tseg, B);
     }
     static void overlap(const RunDesc* d, const OverlapDesc* od, int grid, int wpb,
                         unsigned table, cudaStream_t s) {

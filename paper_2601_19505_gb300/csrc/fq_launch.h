@@ -35,7 +35,7 @@ struct KernelSet {
     void (*ref_count)(const ModelParams&, const void* refs, int n, unsigned* m, cudaStream_t);
     void (*ref_terms)(const ModelParams&, const void* refs, const double* y, int n,
                       const unsigned* off, void* tkeys, double* th, double* tv, unsigned* tseg,
-                      int log2B, cudaStream_t);
+                      unsigned B, cudaStream_t);
     // replica overlaps: `grid` blocks of `wpb` warps, then the row
     void (*overlap)(const RunDesc* runs, const OverlapDesc* od, int grid, int wpb,
                     unsigned table, cudaStream_t);

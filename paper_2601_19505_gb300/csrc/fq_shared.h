@@ -91,7 +91,6 @@ struct RunDesc {
     int norm_q;         // exact norm unit 2^norm_q
     int trel_one;       // t_rel == 1
     unsigned key_x, key_y;   // Philox key
-    int log2B;
     unsigned B, seg_base, Cv, Cs;
     unsigned Cp;             // spawn slots per bucket in the dense primary region (<= Cs)
     void* vkeys[2];
@@ -157,6 +156,8 @@ struct LaunchCfg {
     int merge_var;        // compiled variant of the merge kernel
     int merge_wpb;        // its warps per block
     int merge_grid;       // persistent merge blocks
+    // a batch's first segment of every warp, and the end (null: equal counts)
+    const unsigned *spawn_cuts, *merge_cuts;
     unsigned slots;       // per merge warp: on-chip hash-table slots (power of 2), or
                           // sort-workspace elements
     unsigned scratch_slots;       // global scratch table slots per merge warp
