@@ -315,7 +315,7 @@ template <int KIND> struct RealModel {
         else val = __ldg(p.hop_tab + ns * (nt + 1));
         return dest;
     }
-    // sum over modes of n (n - 1), so H_ii = (u/2) times this: windows of
+    // half the sum over modes of n (n - 1), so H_ii = u times this: windows of
     // w >= 2 consecutive one-bits lie inside one mode's run, and a run of n
     // ones holds n(n-1)/2 of them
     template <class K> __device__ __forceinline__ static int diag_index(K k) {
@@ -325,7 +325,7 @@ template <int KIND> struct RealModel {
             s += KeyOps<K>::popc(x);
             x &= x >> 1;
         }
-        return 2 * s;
+        return s;
     }
 };
 

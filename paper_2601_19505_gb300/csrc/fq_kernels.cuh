@@ -825,6 +825,22 @@ __device__ __forceinline__ void bucket_finish(const RunDesc* R, unsigned seg, un
     }
 }
 
+// (u/2) sum n(n-1), the sum given by half its value
+__device__ __forceinline__ double half_energy(double u, int half) {
+    return (u * 0.5) * (double)(2 * half);
+}
+
+// The diagonal factor 1 + dt (S - H_ii), or its FP32 increment, of an address
+// with sum n(n-1) = 2 half, from the step's table or (rare) computed.
+template <int AMP>
+__device__ __forceinline__ typename AmpT<AMP>::C diag_factor(const RunDesc* R, const StepConst& kc,
+                                                            int half) {
+    typedef typename AmpT<AMP>::C C;
+    if (half < FQ_FACTORS) return __ldg((const C*)kc.diag + half);
+    const double d = R->st->dt * (R->st->shift - half_energy(R->mp.u, half));
+    return AMP == FQ_AMP_F32 ? (C)d : (C)(1.0 + d);
+}
+
 // The diagonal term of an entry c of c^(n) at `key`: c (1 + dt (S - H_ii))
 // (Eq. stochasticTransitionOperator; integer walkers round it stochastically
 // with the draw of stream 0xFFFFFFFE); under early compression it is then
@@ -837,13 +853,13 @@ __device__ __forceinline__ typename AmpT<AMP>::ACC diag_term(const RunDesc* R, c
     typedef Model<KIND> MD;
     ACC w;
     if constexpr (KIND != FQ_KIND_MOM_1D) {
-        const int si = MD::diag_index(key);
+        const typename AmpT<AMP>::C f = diag_factor<AMP>(R, kc, MD::diag_index(key));
         if constexpr (AMP == FQ_AMP_F32) {
-            w = c + c * __ldg((const float*)kc.diag + si);
+            w = c + c * f;
         } else if constexpr (AMP == FQ_AMP_F64) {
-            w = c * __ldg((const double*)kc.diag + si);
+            w = c * f;
         } else {
-            const double x = (double)c * __ldg((const double*)kc.diag + si);
+            const double x = (double)c * f;
             const double fl = floor(x);
             const uint4 r4 = draw(rkey, stepno, 0xFFFFFFFEu, KeyOps<K>::rng_h(key));
             w = (ACC)((long long)fl + (uniform53(r4) < x - fl ? 1 : 0));
@@ -1322,13 +1338,14 @@ __global__ void k_scratch_init(unsigned char* scratch, unsigned SS, unsigned nwa
 
 // ---------------------------------------------------------------------------
 // diagonal factors of the coming step: 1 + dt (S - H_ii) and its FP32
-// increment, per value s = sum n(n-1) (real space, H_ii = (u/2) s)
+// increment, per half = sum n(n-1) / 2 (real space, H_ii = (u/2) 2 half), for
+// the FQ_FACTORS smallest; the few addresses beyond compute theirs
 
 __device__ __forceinline__ void write_factors(const RunDesc* R, double S, double dt) {
-    for (int s = threadIdx.x; s <= R->smax; s += blockDim.x) {
-        const double hii = (R->mp.u * 0.5) * (double)s;
-        R->fac64[s] = 1.0 + dt * (S - hii);
-        R->del32[s] = (float)(dt * (S - hii));
+    for (int i = threadIdx.x; i < FQ_FACTORS; i += blockDim.x) {
+        const double hii = half_energy(R->mp.u, i);
+        R->fac64[i] = 1.0 + dt * (S - hii);
+        R->del32[i] = (float)(dt * (S - hii));
     }
 }
 
@@ -1337,7 +1354,7 @@ __device__ __forceinline__ void write_factors(const RunDesc* R, double S, double
 static __global__ void k_factors(const RunDesc* __restrict__ runs) {
     const RunDesc* R = runs + blockIdx.x;
     const double dt = R->st->dt;
-    if (R->smax >= 0 && R->fac64) write_factors(R, R->st->shift, dt);
+    if (R->fac64) write_factors(R, R->st->shift, dt);
     if (R->coef64) {
         const int w = R->mmax + 1;
         const float dtf = (float)dt;
@@ -1350,87 +1367,112 @@ static __global__ void k_factors(const RunDesc* __restrict__ runs) {
 }
 
 // ---------------------------------------------------------------------------
-// K5: shift update (Eq. shift-update), one block per run
+// K5: shift update (Eq. shift-update), one block per run.  A chain of
+// latencies: partials from L2, a tree, a quotient and a logarithm, the factor
+// table.  The state is read while the partials arrive, the tree's last levels
+// are shuffles, two lanes compute the two quotients and logarithms side by
+// side, and the table holds the factors that occur: the whole table of N = 64
+// (4033 entries, one per sum n(n-1)) took as long as the rest, FP64 being the
+// scarce unit (8.5 us at N = 12..33 and 15-17 at N = 64 before; a step is 1-2 us
+// shorter with this form, 6 at N = 64).
 
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK) k_shift(const RunDesc* __restrict__ runs) {
     const RunDesc* R = runs + blockIdx.x;
     RunState* st = R->st;
-    __shared__ double s_S;
+    __shared__ double s_S, s_dt;
     __shared__ int s_ok;
     __shared__ double s_h[BLOCK], s_v[BLOCK];
+    const int t = threadIdx.x;
+    double nrm = 0.0, rel = 0.0, damp = 0.0, dt = 0.0, shift = 0.0;
+    unsigned long long len = 0;
+    unsigned err = 0;
+    if (t < 32) {
+        err = *(volatile unsigned*)&st->err;
+        len = st->len_acc;
+        dt = st->dt;
+        shift = st->shift;
+        // lane 1: the forcing towards the target; the others: the damping
+        rel = t == 1 ? st->target : st->norm;
+        damp = t == 1 ? st->xi : st->zeta;
+        nrm = R->mode_det ? st->norm_fp : fixed_to_double(st->norm_lo, st->norm_hi, R->norm_q);
+    }
     // the projected-energy partials of the reference buckets: strided over
     // the block, then a tree in a fixed order (the result does not depend on
     // timing)
-    {
-        double hp = 0.0, vp = 0.0;
-        for (unsigned i = threadIdx.x; i < R->n_ref_bkt; i += BLOCK) {
-            const unsigned b = R->ref_bkt[i];
-            hp += R->part_h[b];
-            vp += R->part_v[b];
-        }
-        s_h[threadIdx.x] = hp;
-        s_v[threadIdx.x] = vp;
-        __syncthreads();
-        for (int o = BLOCK / 2; o > 0; o >>= 1) {
-            if ((int)threadIdx.x < o) {
-                s_h[threadIdx.x] += s_h[threadIdx.x + o];
-                s_v[threadIdx.x] += s_v[threadIdx.x + o];
-            }
-            __syncthreads();
-        }
+    double hp = 0.0, vp = 0.0;
+    for (unsigned i = t; i < R->n_ref_bkt; i += BLOCK) {
+        const unsigned b = R->ref_bkt[i];
+        hp += R->part_h[b];
+        vp += R->part_v[b];
     }
-    if (threadIdx.x == 0) {
-        s_ok = 0;
-        if (!*(volatile unsigned*)&st->err) {
-            double nrm;
-            if (R->mode_det) nrm = st->norm_fp;
-            else nrm = fixed_to_double(st->norm_lo, st->norm_hi, R->norm_q);
-            const unsigned long long len = st->len_acc;
-            const double hp = s_h[0], vp = s_v[0];
-            if (nrm == 0.0 || len == 0) {
-                st->err |= FQ_DERR_EMPTY;
-            } else {
-                const double dt = st->dt;
-                const double zd = st->zeta / dt, xd = st->xi / dt;
-                const double S1 =
-                    (st->shift - zd * log(nrm / st->norm)) - xd * log(nrm / st->target);
-                StatsRow row;
-                row.step = st->step + 1;
-                row.len = (long long)len;
-                row.exact_steps = (long long)st->n_exact;
-                row.inexact_steps = (long long)st->n_inexact;
-                row.n_spawns = (long long)st->n_spawns;
-                row.shift = S1;
-                row.norm = nrm;
-                row.hproj = hp;
-                row.vproj = vp;
-                R->hist[st->hist_head % FQ_HIST_CAP] = row;
-                st->hist_head += 1;
-                st->shift = S1;
-                st->norm = nrm;
-                st->step += 1;
-                st->len = (long long)len;
-                st->cur ^= 1;
-                st->last_hproj = hp;
-                st->last_vproj = vp;
-                st->last_exact = row.exact_steps;
-                st->last_inexact = row.inexact_steps;
-                st->last_spawns = row.n_spawns;
-                s_S = S1;
-                s_ok = 1;
+    s_h[t] = hp;
+    s_v[t] = vp;
+    __syncthreads();
+    for (int o = BLOCK / 2; o >= 32; o >>= 1) {
+        if (t < o) {
+            s_h[t] += s_h[t + o];
+            s_v[t] += s_v[t + o];
+        }
+        __syncthreads();
+    }
+    if (t < 32) {
+        hp = s_h[t];
+        vp = s_v[t];
+        for (int o = 16; o > 0; o >>= 1) {
+            const double h = __shfl_down_sync(0xFFFFFFFFu, hp, o);
+            const double v = __shfl_down_sync(0xFFFFFFFFu, vp, o);
+            hp += h;
+            vp += v;
+        }
+        // S - (zeta/dt) log(N'/N) - (xi/dt) log(N'/N_t)
+        const double term = (damp / dt) * log(nrm / rel);
+        const double forcing = __shfl_sync(0xFFFFFFFFu, term, 1);
+        if (t == 0) {
+            s_ok = 0;
+            if (!err) {
+                if (nrm == 0.0 || len == 0) {
+                    st->err |= FQ_DERR_EMPTY;
+                } else {
+                    const double S1 = (shift - term) - forcing;
+                    StatsRow row;
+                    row.step = st->step + 1;
+                    row.len = (long long)len;
+                    row.exact_steps = (long long)st->n_exact;
+                    row.inexact_steps = (long long)st->n_inexact;
+                    row.n_spawns = (long long)st->n_spawns;
+                    row.shift = S1;
+                    row.norm = nrm;
+                    row.hproj = hp;
+                    row.vproj = vp;
+                    R->hist[st->hist_head % FQ_HIST_CAP] = row;
+                    st->hist_head += 1;
+                    st->shift = S1;
+                    st->norm = nrm;
+                    st->step += 1;
+                    st->len = (long long)len;
+                    st->cur ^= 1;
+                    st->last_hproj = hp;
+                    st->last_vproj = vp;
+                    st->last_exact = row.exact_steps;
+                    st->last_inexact = row.inexact_steps;
+                    st->last_spawns = row.n_spawns;
+                    s_S = S1;
+                    s_dt = dt;
+                    s_ok = 1;
+                }
+                st->n_exact = 0;
+                st->n_inexact = 0;
+                st->n_spawns = 0;
+                st->norm_lo = 0;
+                st->norm_hi = 0;
+                st->norm_fp = 0.0;
+                st->len_acc = 0;
             }
-            st->n_exact = 0;
-            st->n_inexact = 0;
-            st->n_spawns = 0;
-            st->norm_lo = 0;
-            st->norm_hi = 0;
-            st->norm_fp = 0.0;
-            st->len_acc = 0;
         }
     }
     __syncthreads();
-    if (s_ok && R->smax >= 0 && R->fac64) write_factors(R, s_S, st->dt);
+    if (s_ok && R->fac64) write_factors(R, s_S, s_dt);
 }
 
 // ---------------------------------------------------------------------------
