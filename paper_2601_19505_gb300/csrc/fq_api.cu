@@ -102,6 +102,7 @@ struct fq_run {
     unsigned* sfill;
     double *part_h, *part_v;
     Tables tab;
+    int nfac;              // factor table: one entry per sum n(n-1) / 2
     double* fac64;
     float* del32;
     RunDesc* d_self;       // this run's descriptor in device memory
@@ -518,6 +519,7 @@ static void fill_desc(const fq_run* r, RunDesc& d, unsigned seg_base) {
     d.mmax = r->tab.mmax;
     d.coef64 = r->tab.r64;
     d.coef32 = r->tab.r32;
+    d.nfac = r->nfac;
     d.fac64 = r->fac64;
     d.del32 = r->del32;
     d.ref_bkt = r->ref_bkt;
@@ -760,9 +762,10 @@ extern "C" int fq_run_create(fq_run** out, const fq_ham* h, const fq_params* p, 
     const size_t nrat = mp0.kind == FQ_BH_MOM_1D ? 0 : (size_t)(r->tab.mmax + 1) * (r->tab.mmax + 1);
     r->tab.r64 = nrat ? (double*)A(sizeof(double) * nrat) : nullptr;
     r->tab.r32 = nrat ? (float*)A(sizeof(float) * nrat) : nullptr;
-    const bool real = mp0.kind != FQ_BH_MOM_1D;
-    r->fac64 = real ? (double*)A(sizeof(double) * FQ_FACTORS) : nullptr;
-    r->del32 = real ? (float*)A(sizeof(float) * FQ_FACTORS) : nullptr;
+    r->nfac = mp0.kind == FQ_BH_MOM_1D ? 0 : mp0.N * (mp0.N - 1) / 2 + 1;
+    const bool f32 = r->amp == FQ_AMP_F32;
+    r->fac64 = r->nfac && !f32 ? (double*)A(sizeof(double) * r->nfac) : nullptr;
+    r->del32 = r->nfac && f32 ? (float*)A(sizeof(float) * r->nfac) : nullptr;
     r->d_self = (RunDesc*)A(sizeof(RunDesc));
     r->ref_cap = 0;
     r->ref_keys = nullptr;
@@ -901,7 +904,7 @@ extern "C" int fq_run_seed(fq_run* r, const fq_key* keys, const double* amps, si
         r->ks->seed(r->d_self, d_k, d_a, m, r->stream);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess && r->fac64) {
+    if (e == cudaSuccess && r->nfac) {
         launch_factors(r->d_self, 1, r->stream);
         e = cudaGetLastError();
     }
@@ -1031,7 +1034,7 @@ static int set_state_field(fq_run* r, size_t offset, double v) {
     CK(cudaMemcpyAsync((char*)r->st + offset, r->pinned, sizeof(double), cudaMemcpyHostToDevice,
                        r->stream));
     CK(cudaEventRecord(r->staged, r->stream));
-    if (r->fac64 && (offset == offsetof(RunState, shift) || offset == offsetof(RunState, dt))) {
+    if (r->nfac && (offset == offsetof(RunState, shift) || offset == offsetof(RunState, dt))) {
         launch_factors(r->d_self, 1, r->stream);
         CK(cudaGetLastError());
     }

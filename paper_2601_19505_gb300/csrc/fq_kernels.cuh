@@ -825,22 +825,6 @@ __device__ __forceinline__ void bucket_finish(const RunDesc* R, unsigned seg, un
     }
 }
 
-// (u/2) sum n(n-1), the sum given by half its value
-__device__ __forceinline__ double half_energy(double u, int half) {
-    return (u * 0.5) * (double)(2 * half);
-}
-
-// The diagonal factor 1 + dt (S - H_ii), or its FP32 increment, of an address
-// with sum n(n-1) = 2 half, from the step's table or (rare) computed.
-template <int AMP>
-__device__ __forceinline__ typename AmpT<AMP>::C diag_factor(const RunDesc* R, const StepConst& kc,
-                                                            int half) {
-    typedef typename AmpT<AMP>::C C;
-    if (half < FQ_FACTORS) return __ldg((const C*)kc.diag + half);
-    const double d = R->st->dt * (R->st->shift - half_energy(R->mp.u, half));
-    return AMP == FQ_AMP_F32 ? (C)d : (C)(1.0 + d);
-}
-
 // The diagonal term of an entry c of c^(n) at `key`: c (1 + dt (S - H_ii))
 // (Eq. stochasticTransitionOperator; integer walkers round it stochastically
 // with the draw of stream 0xFFFFFFFE); under early compression it is then
@@ -853,7 +837,8 @@ __device__ __forceinline__ typename AmpT<AMP>::ACC diag_term(const RunDesc* R, c
     typedef Model<KIND> MD;
     ACC w;
     if constexpr (KIND != FQ_KIND_MOM_1D) {
-        const typename AmpT<AMP>::C f = diag_factor<AMP>(R, kc, MD::diag_index(key));
+        typedef typename AmpT<AMP>::C C;
+        const C f = __ldg((const C*)kc.diag + MD::diag_index(key));
         if constexpr (AMP == FQ_AMP_F32) {
             w = c + c * f;
         } else if constexpr (AMP == FQ_AMP_F64) {
@@ -1337,15 +1322,18 @@ __global__ void k_scratch_init(unsigned char* scratch, unsigned SS, unsigned nwa
 }
 
 // ---------------------------------------------------------------------------
-// diagonal factors of the coming step: 1 + dt (S - H_ii) and its FP32
-// increment, per half = sum n(n-1) / 2 (real space, H_ii = (u/2) 2 half), for
-// the FQ_FACTORS smallest; the few addresses beyond compute theirs
+// diagonal factors of the coming step, per half = sum n(n-1) / 2 (real space,
+// H_ii = (u/2) 2 half): 1 + dt (S - H_ii), or for FP32 amplitudes its FP32
+// increment.  One block writes the table every step, and FP64 is the scarce
+// unit: only what the run's amplitudes read, and only sums that occur (the odd
+// ones never do).
 
 __device__ __forceinline__ void write_factors(const RunDesc* R, double S, double dt) {
-    for (int i = threadIdx.x; i < FQ_FACTORS; i += blockDim.x) {
-        const double hii = half_energy(R->mp.u, i);
-        R->fac64[i] = 1.0 + dt * (S - hii);
-        R->del32[i] = (float)(dt * (S - hii));
+    const double u2 = R->mp.u * 0.5;
+    for (int i = threadIdx.x; i < R->nfac; i += blockDim.x) {
+        const double d = dt * (S - u2 * (double)(2 * i));
+        if (R->amp == FQ_AMP_F32) R->del32[i] = (float)d;
+        else R->fac64[i] = 1.0 + d;
     }
 }
 
@@ -1354,7 +1342,7 @@ __device__ __forceinline__ void write_factors(const RunDesc* R, double S, double
 static __global__ void k_factors(const RunDesc* __restrict__ runs) {
     const RunDesc* R = runs + blockIdx.x;
     const double dt = R->st->dt;
-    if (R->fac64) write_factors(R, R->st->shift, dt);
+    if (R->nfac) write_factors(R, R->st->shift, dt);
     if (R->coef64) {
         const int w = R->mmax + 1;
         const float dtf = (float)dt;
@@ -1371,10 +1359,10 @@ static __global__ void k_factors(const RunDesc* __restrict__ runs) {
 // latencies: partials from L2, a tree, a quotient and a logarithm, the factor
 // table.  The state is read while the partials arrive, the tree's last levels
 // are shuffles, two lanes compute the two quotients and logarithms side by
-// side, and the table holds the factors that occur: the whole table of N = 64
-// (4033 entries, one per sum n(n-1)) took as long as the rest, FP64 being the
-// scarce unit (8.5 us at N = 12..33 and 15-17 at N = 64 before; a step is 1-2 us
-// shorter with this form, 6 at N = 64).
+// side, and the table holds half as many factors of one kind instead of both.
+// Before: 8.5 us at N = 12..33, 15-17 at N = 64; 3 to 6 us less now.  (A table of 256
+// entries, the merge computing the rare factors beyond, was shorter still
+// here, but that branch cost the merge 7 %: 480 -> 516 us at 1e7 walkers.)
 
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK) k_shift(const RunDesc* __restrict__ runs) {
@@ -1472,7 +1460,7 @@ __global__ void __launch_bounds__(BLOCK) k_shift(const RunDesc* __restrict__ run
         }
     }
     __syncthreads();
-    if (s_ok && R->fac64) write_factors(R, s_S, s_dt);
+    if (s_ok && R->nfac) write_factors(R, s_S, s_dt);
 }
 
 // ---------------------------------------------------------------------------

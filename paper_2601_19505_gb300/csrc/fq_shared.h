@@ -28,7 +28,6 @@
 #define FQ_ANN_SORT_ARM 1
 
 #define FQ_MAX_MOM_MODES 64
-#define FQ_FACTORS 256  // entries of a run's table of diagonal factors
 #define FQ_HIST_CAP 65536u
 
 namespace fq {
@@ -105,8 +104,9 @@ struct RunDesc {
     int mmax;                 // largest m of the coefficient tables (real space)
     double* coef64;           // (-dt) ((double)m / (double)n), index m * (mmax + 1) + n
     float* coef32;            // the same in FP32 arithmetic
-    double* fac64;            // 1 + dt (S - H_ii) per sum n(n-1) / 2 < FQ_FACTORS, this step
-    float* del32;             // (float)(dt (S - H_ii)), the same (both null in momentum space)
+    int nfac;                 // entries of the factor table (0 in momentum space)
+    double* fac64;            // 1 + dt (S - H_ii) per sum n(n-1) / 2, this step
+    float* del32;             // (float)(dt (S - H_ii)), the same (FP32 amplitudes; else null)
     const void* ref_keys;     // reference terms sorted by segment
     const double* ref_h;      // y_r H_{r,j}
     const double* ref_v;      // y_r on the reference address itself, else 0

@@ -1,6 +1,5 @@
-"""Diagonal factors of addresses beyond the step's factor table (sum n(n-1) / 2
-of 256 and more, condensates in real space) follow the oracle like those in it
-(needs a GB300)."""
+"""Diagonal factors over the whole range of sum n(n-1) / 2, condensates in real
+space included, follow the oracle (needs a GB300)."""
 import numpy as np
 import pytest
 
@@ -17,7 +16,7 @@ def test_condensed_addresses_match_oracle(model, mode):
     h, m = pair(*model)
     N, M = model[3], model[1] * model[2]
     occs = []
-    for top in (N, N - 1, 24, 23, 22, 5):  # 23 bosons on a site: half the sum is 253
+    for top in (N, N - 1, 24, 23, 22, 5):
         occ = np.zeros(M, dtype=np.uint8)
         occ[0] = top
         occ[1] += (N - top) // 2
