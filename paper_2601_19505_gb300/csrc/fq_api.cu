@@ -51,8 +51,8 @@ const KernelSet* kernel_set(int kw, int amp, int kind) {
     return &g_sets[kw - 1][amp][kind - 1];
 }
 
-void launch_shift(const RunDesc* runs, int nruns, cudaStream_t s) {
-    k_shift<256><<<nruns, 256, 0, s>>>(runs);
+void launch_shift(const RunDesc* runs, int nruns, int early, cudaStream_t s) {
+    launch_after(early, k_shift<256>, nruns, 256, 0, s, runs);
 }
 
 static void launch_factors(const RunDesc* runs, int nruns, cudaStream_t s) {
@@ -1070,7 +1070,7 @@ static void enqueue_steps(fq_batch* b, int n, cudaStream_t s) {
         b->ks->spawn(b->cfg, b->d_desc, b->d_seg_run, b->G, s);
         b->ks->merge(b->cfg, b->d_desc, b->d_seg_run, b->G, s);
         launch_gs(b, s);
-        launch_shift(b->d_desc, nr, s);
+        launch_shift(b->d_desc, nr, b->cfg.early_launch, s);
         launch_overlaps(b, s);
     }
 }
@@ -1328,11 +1328,13 @@ static int batch_build(fq_batch* b) {
     std::vector<RunDesc> desc(nr);
     std::vector<unsigned> seg_run;
     unsigned base = 0, slots = 0, ss = 0, se = 0;
+    double spawns = 0.0;  // expected per step
     for (size_t i = 0; i < nr; ++i) {
         fq_run* r = b->runs[i];
         fill_desc(r, desc[i], base);
         for (unsigned s = 0; s < r->B; ++s) seg_run.push_back((unsigned)i);
         base += r->B;
+        spawns += r->fill * r->B;
         slots = std::max(slots, r->slots);
         ss = std::max(ss, r->scratch_slots);
         se = std::max(se, r->sort_elems);
@@ -1396,6 +1398,7 @@ static int batch_build(fq_batch* b) {
     }
     for (LaunchCfg& c : b->shapes) {
         c.scratch = b->scratch;
+        c.early_launch = spawns <= kEarlySpawns;
         c.scratch_slots = ss;
         c.sort_scratch = b->sort_scratch;
         c.sort_elems = se;
@@ -1878,7 +1881,7 @@ static int autotune(fq_batch* b, int steps) {
         b->ks->merge(c, b->d_desc, b->d_seg_run, b->G, b->stream);
         e = cudaEventRecord(ev[3 * t + 2], b->stream);
         launch_gs(b, b->stream);
-        launch_shift(b->d_desc, nr, b->stream);
+        launch_shift(b->d_desc, nr, 0, b->stream);
         launch_overlaps(b, b->stream);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
@@ -1972,7 +1975,7 @@ extern "C" int fq_run_profile(fq_run* r, int n, float* ms) {
         cudaEventRecord(ev[4 * i + 1], r->stream);
         b->ks->merge(b->cfg, b->d_desc, b->d_seg_run, b->G, r->stream);
         cudaEventRecord(ev[4 * i + 2], r->stream);
-        launch_shift(b->d_desc, 1, r->stream);
+        launch_shift(b->d_desc, 1, 0, r->stream);
         e = cudaEventRecord(ev[4 * i + 3], r->stream);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(r->stream);

@@ -219,6 +219,21 @@ __device__ __forceinline__ void warp_copy_async(void* dst, const void* src, unsi
 }
 
 // ---------------------------------------------------------------------------
+// Programmatic dependent launch: the kernels of a step are launched without a
+// wait for the one before (launch_after in fq_launch.h).  Each lets the next
+// one's blocks start as soon as it has begun itself, does what does not depend
+// on the step before it (descriptors, parameters, empty tables), and waits
+// here for the kernel before it to have finished and its writes to be visible.
+// Every thread waits, also those without work, so that a kernel never ends
+// before the one before it and the chain of dependences holds through it.
+__device__ __forceinline__ void let_next_start() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void wait_for_previous() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// ---------------------------------------------------------------------------
 // K1: spawning.  One warp per segment range; a segment is taken in batches
 // of up to 32 * IPT entries, staged in shared memory by cp.async one batch
 // ahead, each lane owning IPT consecutive entries; the batch's spawn
@@ -271,11 +286,19 @@ k_spawn(const RunDesc* __restrict__ runs, const unsigned* __restrict__ seg_run, 
     const ModelParams& mp = *wmp;
     unsigned g0, g1;
     warp_range(cuts, G, blockIdx.x * WPB + wib, gridDim.x * WPB, g0, g1);
-    if (g0 >= g1) return;  // fewer segments than warps
+    let_next_start();
+    if (g0 >= g1) {  // fewer segments than warps
+        wait_for_previous();
+        return;
+    }
 
     // the range's run (a range never crosses runs): its first segment and
     // per-step constants
     const RunDesc* const R = runs + seg_run[g0];
+    for (unsigned i = (unsigned)lane; i < (unsigned)(SM::mp_bytes / 4); i += 32u)
+        ((unsigned*)wmp)[i] = ((const unsigned*)&R->mp)[i];
+    __syncwarp();
+    wait_for_previous();
     // lane 0 reads, the warp shares: another warp may set an error bit
     unsigned err = 0, cur = 0;
     if (lane == 0) {
@@ -303,9 +326,6 @@ k_spawn(const RunDesc* __restrict__ runs, const unsigned* __restrict__ seg_run, 
     const typename AmpT<AMP>::C* r_coef = nullptr;
     if constexpr (AMP == FQ_AMP_F32) r_coef = R->coef32;
     else if constexpr (AMP == FQ_AMP_F64) r_coef = R->coef64;
-    for (unsigned i = (unsigned)lane; i < (unsigned)(SM::mp_bytes / 4); i += 32u)
-        ((unsigned*)wmp)[i] = ((const unsigned*)&R->mp)[i];
-    __syncwarp();
     unsigned n_ex = 0, n_inex = 0, n_sp = 0;
 
     // the spawn whose bucket slot is being reserved (stored one spawn later)
@@ -1194,6 +1214,8 @@ k_merge(const RunDesc* __restrict__ runs, const unsigned* __restrict__ seg_run, 
     unsigned g0, g1;
     warp_range(cuts, G, gw, gridDim.x * WPB, g0, g1);
 
+    let_next_start();
+    wait_for_previous();
     if (g0 >= g1) return;
     // The range's run: a range never crosses runs.  (A loop over the runs of a
     // range, with totals flushed and restarted between them, counted wrongly
@@ -1372,6 +1394,8 @@ __global__ void __launch_bounds__(BLOCK) k_shift(const RunDesc* __restrict__ run
     __shared__ int s_ok;
     __shared__ double s_h[BLOCK], s_v[BLOCK];
     const int t = threadIdx.x;
+    let_next_start();
+    wait_for_previous();
     double nrm = 0.0, rel = 0.0, damp = 0.0, dt = 0.0, shift = 0.0;
     unsigned long long len = 0;
     unsigned err = 0;

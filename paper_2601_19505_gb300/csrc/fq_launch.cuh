@@ -18,8 +18,8 @@ template <class K, int AMP, int KIND> struct Launch {
     template <int V> static void spawn_v(const LaunchCfg& c, const RunDesc* d, const unsigned* sr,
                                          unsigned G, cudaStream_t s) {
         constexpr int W = Var<V>::WPB;
-        k_spawn<K, AMP, KIND, V, 4><<<c.spawn_grid, W * 32, spawn_smem(W), s>>>(d, sr, G,
-                                                                                  c.spawn_cuts);
+        launch_after(c.early_launch, k_spawn<K, AMP, KIND, V, 4>, c.spawn_grid, W * 32, spawn_smem(W), s, d, sr, G,
+                     c.spawn_cuts);
     }
     static void spawn(const LaunchCfg& c, const RunDesc* d, const unsigned* sr, unsigned G,
                       cudaStream_t s) {
@@ -32,12 +32,12 @@ template <class K, int AMP, int KIND> struct Launch {
         constexpr int W = Var<V>::WPB;
         if (c.ann == FQ_ANN_SORT_ARM) {
             const size_t smem = (size_t)W * merge_warp_bytes<K, AMP, FQ_ANN_SORT_ARM>(c.slots);
-            k_merge<K, AMP, KIND, V, FQ_ANN_SORT_ARM><<<c.merge_grid, W * 32, smem, s>>>(
-                d, sr, G, c.slots, c.sort_scratch, c.sort_elems, c.merge_cuts);
+            launch_after(c.early_launch, k_merge<K, AMP, KIND, V, FQ_ANN_SORT_ARM>, c.merge_grid, W * 32, smem, s, d,
+                         sr, G, c.slots, c.sort_scratch, c.sort_elems, c.merge_cuts);
         } else {
             const size_t smem = (size_t)W * merge_warp_bytes<K, AMP, FQ_ANN_HASH_ARM>(c.slots);
-            k_merge<K, AMP, KIND, V, FQ_ANN_HASH_ARM><<<c.merge_grid, W * 32, smem, s>>>(
-                d, sr, G, c.slots, c.scratch, c.scratch_slots, c.merge_cuts);
+            launch_after(c.early_launch, k_merge<K, AMP, KIND, V, FQ_ANN_HASH_ARM>, c.merge_grid, W * 32, smem, s, d,
+                         sr, G, c.slots, c.scratch, c.scratch_slots, c.merge_cuts);
         }
     }
     static void merge(const LaunchCfg& c, const RunDesc* d, const unsigned* sr, unsigned G,

@@ -156,6 +156,7 @@ struct LaunchCfg {
     int merge_var;        // compiled variant of the merge kernel
     int merge_wpb;        // its warps per block
     int merge_grid;       // persistent merge blocks
+    int early_launch;     // the step's kernels may start before the one before them ends
     // a batch's first segment of every warp, and the end (null: equal counts)
     const unsigned *spawn_cuts, *merge_cuts;
     unsigned slots;       // per merge warp: on-chip hash-table slots (power of 2), or
