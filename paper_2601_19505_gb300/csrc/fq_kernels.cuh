@@ -452,6 +452,11 @@ k_spawn(const RunDesc* __restrict__ runs, const unsigned* __restrict__ seg_run, 
         unsigned xoff = 0;
         for (int j = 0; j < IPT; ++j) {
             const unsigned i = (unsigned)j * 32u + (unsigned)lane;
+            // a round without a source (the end of a segment, or a small one)
+            if ((unsigned)j * 32u >= cn) {
+                woff[i] = xoff;
+                continue;
+            }
             unsigned cnt = 0, mm = 0;
             CO cf = (CO)0;
             K key = KeyOps<K>::empty();
