@@ -61,7 +61,7 @@ static void launch_factors(const RunDesc* runs, int nruns, cudaStream_t s) {
 
 // tables of sqrt(k), hop values and m / n for a model (device memory)
 struct Tables {
-    double *sq, *hop, *r64;
+    double *sq, *hop, *r64, *eps;
     float *hop32, *r32;
     int kmax, mmax;
 };
@@ -496,6 +496,7 @@ static ModelParams run_mp(const fq_run* r) {
     mp.sqrt_tab = r->tab.sq;
     mp.hop_tab = r->tab.hop;
     mp.hop32_tab = r->tab.hop32;
+    mp.eps_tab = r->tab.eps;
     return mp;
 }
 
@@ -759,6 +760,8 @@ extern "C" int fq_run_create(fq_run** out, const fq_ham* h, const fq_params* p, 
     r->tab.sq = (double*)A(sizeof(double) * (r->tab.kmax + 1));
     r->tab.hop = (double*)A(sizeof(double) * (r->tab.kmax + 1));
     r->tab.hop32 = (float*)A(sizeof(float) * (r->tab.kmax + 1));
+    const size_t neps = mp0.kind == FQ_BH_MOM_1D ? (size_t)mp0.M * (mp0.N + 1) : 0;
+    r->tab.eps = neps ? (double*)A(sizeof(double) * neps) : nullptr;
     const size_t nrat = mp0.kind == FQ_BH_MOM_1D ? 0 : (size_t)(r->tab.mmax + 1) * (r->tab.mmax + 1);
     r->tab.r64 = nrat ? (double*)A(sizeof(double) * nrat) : nullptr;
     r->tab.r32 = nrat ? (float*)A(sizeof(float) * nrat) : nullptr;
@@ -795,6 +798,12 @@ extern "C" int fq_run_create(fq_run** out, const fq_ham* h, const fq_params* p, 
             h->mp.t, r->tab.kmax, r->tab.sq, r->tab.hop, r->tab.hop32);
         e = cudaGetLastError();
     }
+    std::vector<double> eps(neps);
+    for (size_t i = 0; i < neps; ++i)
+        eps[i] = mp0.eps[i / (mp0.N + 1)] * (double)(i % (mp0.N + 1));
+    if (e == cudaSuccess && neps)
+        e = cudaMemcpyAsync(r->tab.eps, eps.data(), sizeof(double) * neps, cudaMemcpyHostToDevice,
+                            r->stream);
     if (e == cudaSuccess) {
         RunDesc hd;
         fill_desc(r, hd, 0);

@@ -875,7 +875,7 @@ __device__ __forceinline__ typename AmpT<AMP>::ACC diag_term(const RunDesc* R, c
             w = (ACC)((long long)fl + (uniform53(r4) < x - fl ? 1 : 0));
         }
     } else {
-        const double hii = MD::diagonal(R->mp, key);
+        const double hii = MD::template diagonal<K, true>(R->mp, key);
         const double S0 = R->st->shift, dt = R->st->dt;
         if constexpr (AMP == FQ_AMP_F32) {
             w = c + c * (float)(dt * (S0 - hii));

@@ -40,6 +40,7 @@ struct ModelParams {
     const double* sqrt_tab;          // sqrt((double)k), k <= kmax (device)
     const double* hop_tab;           // -(t * sqrt((double)k)), k <= kmax (device)
     const float* hop32_tab;          // (float) of hop_tab
+    const double* eps_tab;           // momentum space: eps[s] n, index s (N + 1) + n (device)
     unsigned char nbr[4][128];       // real space: neighbour of site s in direction d
     // kept last: the spawn kernel copies the members before it for real-space
     // models and the whole struct for momentum space
