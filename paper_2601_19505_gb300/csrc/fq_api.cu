@@ -624,8 +624,8 @@ static double full_segments(double s_ss, unsigned slots) {
 // of the warps that are resident at once (16 per SM in the default launch
 // shape), so that every warp takes the same number: with a power of two, 1e6
 // walkers were 8192 buckets on 2432 warps, where some took four and most
-// three (now 7296: 8 % off the step), and 1e8 walkers 2^20 of 117 spawns
-// instead of 642048 of 171 (2 %).  Below one full bucket per warp, smaller
+// three (now 7296: 8 % off the step), and 1e8 walkers 2^20 of 105 spawns
+// instead of 646912 of 170 (2 %).  Below one full bucket per warp, smaller
 // buckets on more warps, down to one round of 32 spawns: a step of 1e4
 // walkers on 12 sites took 39 us with buckets of 86 spawns and takes 33 with
 // 32, 1e5 on 20 sites 42 and 37.  Less than 64 such buckets (2000 walkers, in
