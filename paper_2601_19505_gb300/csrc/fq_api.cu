@@ -1256,11 +1256,36 @@ static std::vector<int> batch_arms(const fq_batch* b) {
     return {FQ_ANN_HASH_ARM, FQ_ANN_SORT_ARM};
 }
 
+// The shape a batch steps with unless the autotuner finds another.  With many
+// buckets for every warp, more warps of fewer registers: 64-bit addresses
+// spawn with 24 warps per SM (1e7 walkers on 20 sites 334 -> 298 us) and merge
+// with 20 (479 -> 432), 128-bit ones spawn with 20 in two waves of blocks
+// (1e8 walkers on 8 x 8 3277 -> 3111) but merge with 16, as does momentum
+// space (its diagonal wants the registers), which spawns with 24 warps in two
+// waves from one bucket a warp on (1e6 walkers on 32 modes 145 -> 137).  With
+// a few buckets a warp, the segments are cut for 16 warps per SM
+// (segments_for) and other shapes gained nothing.
+static LaunchCfg default_cfg(const fq_batch* b, unsigned slots, int ann) {
+    const bool wide = b->ks->key_bytes == 16;
+    const bool mom = b->runs[0]->ham.mp.kind == FQ_BH_MOM_1D;
+    const unsigned warps = (unsigned)num_sms() * 16u;
+    int sv = 0, waves = 1, mv = 0;
+    if (b->G >= 16u * warps) {
+        sv = wide && !mom ? 1 : 2;
+        waves = wide || mom ? 2 : 1;
+        mv = !wide && !mom && ann == FQ_ANN_HASH_ARM ? 1 : 0;
+    } else if (mom && b->G >= warps) {
+        sv = 2;
+        waves = 2;
+    }
+    return make_cfg(b->ks, sv, waves, mv, slots, b->G, ann);
+}
+
 static std::vector<LaunchCfg> batch_shapes(fq_batch* b, unsigned slots) {
     std::vector<LaunchCfg> v;
     const size_t limit = 200u * 1024u;
     const std::vector<int> arms = batch_arms(b);
-    v.push_back(make_cfg(b->ks, 0, 1, 0, slots, b->G, arms[0]));
+    v.push_back(default_cfg(b, slots, arms[0]));
     for (int ann : arms)
         for (int sv = 0; sv < kKernelVariants; ++sv)
             for (int waves : {1, 2})

@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 
 import oracle as O
-from gpu_helpers import assert_same_vector, fq, pair, runs
+from gpu_helpers import assert_same_vector, fq, pair, runs, seeded_vector
 
 pytestmark = pytest.mark.gpu
 
@@ -51,3 +51,24 @@ def test_uneven_batch_steps_like_its_runs_alone(targets):
         assert np.array_equal(r.history()["n_spawns"], together[i].history()["n_spawns"])
         r.close()
     b.close()
+
+
+@pytest.mark.parametrize("model,target,wpb", [
+    ((O.REAL_1D, 20, 1, 20, 1.0, 2.0), 8e6, (4, 4)), ((O.REAL_1D, 20, 1, 20, 1.0, 2.0), 6e6, (8, 8)),
+    ((O.REAL_2D, 8, 8, 64, 1.0, 8.0), 8e6, (4, 8)), ((O.MOM_1D, 8, 1, 8, 1.0, 4.0), 8e5, (4, 8)),
+    ((O.MOM_1D, 32, 1, 32, 1.0, 4.0), 8e6, (4, 8))], ids=str)
+def test_default_shapes_match_oracle(model, target, wpb):
+    """The launch shape a run steps with untuned, on both sides of the bucket
+    counts at which it changes (16 buckets a warp; one in momentum space)."""
+    h, m = pair(*model)
+    keys, amps = seeded_vector(m, 2000, 17)
+    g, o = runs(h, m, dt=0.001, target=target, seed=12)
+    g.seed(fq().keys_from_ints(keys), amps, -2.0, step=5)
+    o.seed(keys, amps, -2.0, step=5)
+    g.step(2)
+    o.step(2)
+    s = g.shape()
+    assert (s["spawn_wpb"], s["merge_wpb"]) == wpb
+    assert_same_vector(g.export(), o.export(), rtol=1e-12)
+    assert np.array_equal(g.history()["n_spawns"], o.history()["n_spawns"])
+    g.close()
