@@ -54,7 +54,7 @@ def test_uneven_batch_steps_like_its_runs_alone(targets):
 
 
 @pytest.mark.parametrize("model,target,wpb", [
-    ((O.REAL_1D, 20, 1, 20, 1.0, 2.0), 8e6, (4, 4)), ((O.REAL_1D, 20, 1, 20, 1.0, 2.0), 6e6, (8, 8)),
+    ((O.REAL_1D, 20, 1, 20, 1.0, 2.0), 8e6, (4, 4)), ((O.REAL_1D, 20, 1, 20, 1.0, 2.0), 5.5e6, (8, 8)),
     ((O.REAL_2D, 8, 8, 64, 1.0, 8.0), 8e6, (4, 8)), ((O.MOM_1D, 8, 1, 8, 1.0, 4.0), 8e5, (4, 8)),
     ((O.MOM_1D, 32, 1, 32, 1.0, 4.0), 8e6, (4, 8))], ids=str)
 def test_default_shapes_match_oracle(model, target, wpb):
