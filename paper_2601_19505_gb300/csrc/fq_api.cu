@@ -21,6 +21,7 @@
 #include "fq_kernels.cuh"
 #include "fq_launch.h"
 #include "fq_shared.h"
+#include "fq_shares.h"
 
 using namespace fq;
 
@@ -1297,48 +1298,21 @@ static std::vector<LaunchCfg> batch_shapes(fq_batch* b, unsigned slots) {
     return v;
 }
 
-// Every launch shape's shares of the batch's segments: cuts[w] is warp w's
-// first segment.  A share lies within one run, and no share's expected work is
-// more than the smallest bound for which the warps suffice.  A bucket costs
-// about as much as 32 spawns before its first one (batch of 64 runs with
-// buckets of 32 to 170 spawns: 42.9 ms a chunk with 24, 42.4 with 48, 47.7
-// with 8, 45.6 with 96).
-static std::vector<unsigned> share_cuts(const fq_batch* b, unsigned nw) {
-    const std::vector<fq_run*>& runs = b->runs;
-    auto parts = [](const fq_run* r, double most) {  // shares of run r: at most `most` each
-        const double per = std::max(1.0, std::floor(most / (32.0 + r->fill)));  // segments
-        return (unsigned)std::ceil(r->B / per);
-    };
-    double lo = 0.0, hi = 0.0;
-    for (const fq_run* r : runs) hi = std::max(hi, r->B * (32.0 + r->fill));
-    for (int i = 0; i < 40; ++i) {
-        const double mid = 0.5 * (lo + hi);
-        unsigned long long n = 0;
-        for (const fq_run* r : runs) n += parts(r, mid);
-        (n <= nw ? hi : lo) = mid;
-    }
-    std::vector<unsigned> cuts;
-    unsigned base = 0;
-    for (const fq_run* r : runs) {
-        const unsigned k = parts(r, hi);
-        for (unsigned i = 0; i < k; ++i)
-            cuts.push_back(base + (unsigned)((unsigned long long)r->B * i / k));
-        base += r->B;
-    }
-    cuts.resize(nw + 1, base);  // warps beyond the shares have none
-    return cuts;
-}
-
+// every launch shape's shares of the batch's segments (none for a single run:
+// equal counts)
 static int batch_cuts(fq_batch* b) {
     if (b->runs.size() < 2) return FQ_OK;
-    std::vector<unsigned> all;
+    std::vector<ShareRun> runs;
+    for (const fq_run* r : b->runs) runs.push_back({r->B, r->fill});
+    std::vector<unsigned> all, cuts;
     std::vector<std::pair<unsigned, size_t>> have;  // warps, offset of their cuts
+    bool ok = true;
     auto of = [&](int warps) {
         for (const auto& h : have)
             if (h.first == (unsigned)warps) return h.second;
-        const std::vector<unsigned> c = share_cuts(b, (unsigned)warps);
+        ok &= share_cuts(runs, (unsigned)warps, cuts);
         have.push_back({(unsigned)warps, all.size()});
-        all.insert(all.end(), c.begin(), c.end());
+        all.insert(all.end(), cuts.begin(), cuts.end());
         return have.back().second;
     };
     std::vector<size_t> so, mo;
@@ -1346,6 +1320,7 @@ static int batch_cuts(fq_batch* b) {
         so.push_back(of(c.spawn_grid * c.spawn_wpb));
         mo.push_back(of(c.merge_grid * c.merge_wpb));
     }
+    if (!ok) return FQ_ERR_INVALID;
     CK(cudaMalloc((void**)&b->d_cuts, sizeof(unsigned) * all.size()));
     CK(cudaMemcpy(b->d_cuts, all.data(), sizeof(unsigned) * all.size(), cudaMemcpyHostToDevice));
     for (size_t i = 0; i < b->shapes.size(); ++i) {

@@ -164,8 +164,8 @@ __device__ __forceinline__ void warp_range(unsigned G, unsigned w, unsigned nw, 
     g1 = (unsigned)(((unsigned long long)G * (w + 1)) / nw);
 }
 // ... or between the host's cuts: in a batch of runs whose segments hold
-// unequal work, shares of equal work, each of segments of one run (batch_cuts
-// in fq_api.cu).  With equal counts of segments, a warp among the runs of full
+// unequal work, shares of equal work, each of segments of one run (share_cuts
+// in fq_shares.h).  With equal counts of segments, a warp among the runs of full
 // buckets had up to five times the work of one among the runs of small ones,
 // and a batch of 64 runs of 1e4 to 1e6 walkers took 1.92 ms a step instead of
 // 1.33.
