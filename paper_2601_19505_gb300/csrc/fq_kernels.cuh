@@ -863,7 +863,11 @@ __device__ __forceinline__ typename AmpT<AMP>::ACC diag_term(const RunDesc* R, c
     ACC w;
     if constexpr (KIND != FQ_KIND_MOM_1D) {
         typedef typename AmpT<AMP>::C C;
-        const C f = __ldg((const C*)kc.diag + MD::diag_index(key));
+        // an ordinary load, not __ldg: blocks of this kernel may be resident
+        // while the shift update of the step before writes the table
+        // (wait_for_previous), and read-only loads ask that the data stay as
+        // they are for as long as the kernel runs
+        const C f = ((const C*)kc.diag)[MD::diag_index(key)];
         if constexpr (AMP == FQ_AMP_F32) {
             w = c + c * f;
         } else if constexpr (AMP == FQ_AMP_F64) {
