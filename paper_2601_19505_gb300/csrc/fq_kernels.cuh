@@ -968,6 +968,9 @@ __device__ __forceinline__ void merge_bucket(const RunDesc* R, unsigned seg, uns
             }
             if (nw) tl[nl + __popc(bal & ((1u << lane) - 1u))] = (unsigned)q;
             nl += __popc(bal);
+            // this round's sums before the next round's reads of them (the
+            // votes above order no memory)
+            __syncwarp();
         }
     }
     __syncwarp();
