@@ -316,7 +316,7 @@ int fq_batch_sync(fq_batch *b);
 int fq_batch_autotune(fq_batch *b, int steps);
 
 /* Replica overlaps (Sec. 4.3, Eq. RayleighQuotientReplica): with R = 2..8
- * replicas in one batch (one Hamiltonian, equal sizes; statistically
+ * replicas in one batch (one Hamiltonian and one size class; statistically
  * independent through their run_id), record after every step, for every pair
  * A < B in the order (0,1), (0,2), ..., (1,2), ..., the vector-vector product
  * c_A^T c_B and the vector-operator-vector products c_A^T G2(d_k) c_B of the
@@ -326,12 +326,17 @@ int fq_batch_autotune(fq_batch *b, int steps);
  * of the means of (S_A + S_B)/2 c_A^T c_B and c_A^T c_B (shifts from each
  * run's history).  Each pair's sums over segments are added in a fixed
  * order, so repeated runs give identical rows.  Replaces any earlier
- * setting; FQ_ERR_INVALID for runs of different shapes or sizes. */
+ * setting; FQ_ERR_INVALID for runs of different shapes or size classes.
+ * A run's size class is its expected number of spawns per step at creation
+ * (1.1 target / min(1, threshold); in the deterministic limit every column
+ * entry of the vector) in units of a third of the default on-chip table
+ * (fq_run_shape's slots), rounded up to a power of two: targets 1e4 and 1.9e4
+ * are of one class, 1e4 and 2.1e4 are not. */
 int fq_batch_set_overlaps(fq_batch *b, const int *g2_d, int n_g2);
 /* Excited states (Sec. 2.2): runs 0..K-1 of the batch (2 <= K <= 8; one
- * Hamiltonian and equal sizes; real-valued or deterministic walkers) become
- * step-synchronised spectral states.  After every step's annihilation, run k
- * is orthogonalised to runs 0..k-1 (Gram-Schmidt): c_k <- c_k - sum_j
+ * Hamiltonian and size class, as for the overlaps; real-valued or
+ * deterministic walkers) become step-synchronised spectral states.  After
+ * every step's annihilation, run k is orthogonalised to runs 0..k-1 (Gram-Schmidt): c_k <- c_k - sum_j
  * alpha_j c_j with alpha_j = (c_j^T c_k) / (c_j^T c_j), all alpha_j from the
  * same c_k; each value that changed is then compressed by Pi (Eq.
  * vec-compression, its draw from stream 0xFFFFFFFC of the address), and run
@@ -339,7 +344,7 @@ int fq_batch_set_overlaps(fq_batch *b, const int *g2_d, int n_g2);
  * vector.  The shift of run k estimates the k-th energy (shift_estimator).
  * Seed the runs differently (a later state must not start parallel to an
  * earlier one).  K = 0 turns it off; FQ_ERR_INVALID for integer walkers or
- * runs of different shapes or sizes. */
+ * runs of different shapes or size classes. */
 int fq_batch_set_spectral(fq_batch *b, int K);
 /* Move out the overlap rows recorded since the last call, oldest first, at
  * most cap of them (*n = rows written).  A row is `width` doubles: the step,

@@ -91,6 +91,7 @@ struct fq_run {
     const KernelSet* ks;
     unsigned B, Cv, Cs, slots;  // slots: on-chip table slots per merge warp
     unsigned Cp;                // spawn slots per bucket in the dense primary region
+    unsigned size_class;        // full buckets, rounded up to a power of two (joinable)
     double fill;                // steady-state spawns per bucket
     bool no_spawn_buf;          // a failed growth left no spawn buffers: the run cannot step
     RunState* st;
@@ -716,6 +717,7 @@ extern "C" int fq_run_create(fq_run** out, const fq_ham* h, const fq_params* p, 
         s_ss = l_ss * (double)max_offdiag(h->mp);
     }
     r->B = segments_for(s_ss, r->slots);
+    r->size_class = next_pow2((unsigned long long)full_segments(s_ss, r->slots));
     {
         // spawns arrive in clumps (one address receives spawns from many
         // sources; every neighbour's in the deterministic limit), so the
@@ -1130,7 +1132,16 @@ static int overlaps_build(fq_batch* b) {
     const size_t smem = (size_t)wpb * T * slot;
     CK(b->ks->prepare_overlap(smem));
     const int R = (int)b->runs.size(), P = R * (R - 1) / 2;
-    const unsigned long long items = (unsigned long long)P * b->runs[0]->B;
+    OverlapDesc od;
+    memset(&od, 0, sizeof od);
+    int p = 0;
+    for (int a = 0; a < R; ++a)
+        for (int c = a + 1; c < R; ++c, ++p) {
+            od.pa[p] = a;
+            od.pb[p] = c;
+            od.first[p + 1] = od.first[p] + b->runs[a]->B;
+        }
+    const unsigned long long items = od.first[P];
     b->ov_wpb = wpb;
     b->ov_grid = (int)std::max<unsigned long long>(
         1, std::min<unsigned long long>((unsigned long long)num_sms() * join_blocks_per_sm(smem),
@@ -1144,19 +1155,10 @@ static int overlaps_build(fq_batch* b) {
         CK(cudaMalloc((void**)&b->ov_part, sizeof(double) * need));
         b->ov_part_n = need;
     }
-    OverlapDesc od;
-    memset(&od, 0, sizeof od);
     od.R = R;
     od.P = P;
     od.nq = b->ov_nq;
     for (int k = 0; k < b->ov_nq; ++k) od.d[k] = b->ov_d[k];
-    int p = 0;
-    for (int a = 0; a < R; ++a)
-        for (int c = a + 1; c < R; ++c, ++p) {
-            od.pa[p] = a;
-            od.pb[p] = c;
-        }
-    od.B = b->runs[0]->B;
     od.table = T;
     od.part = b->ov_part;
     od.ring = b->ov_ring;
@@ -1176,19 +1178,28 @@ static void gs_free(fq_batch* b) {
     b->gs_K = 0;
 }
 
-// the Gram-Schmidt launches for the batch's current sizes: one table per
-// warp with more slots than K segments' capacities (an insert always finds one)
+// the Gram-Schmidt launches for the batch's current sizes: one table per warp
+// with more slots than the entries of all K states in a segment of one, at
+// their capacities (an insert finds one; a state of fewer segments than that
+// one could hold more there, and then the step fails as for any full table)
 static int gs_build(fq_batch* b) {
     if (b->gs_K < 2) return FQ_OK;
-    unsigned cv = 0;
-    for (int k = 0; k < b->gs_K; ++k) cv = std::max(cv, b->runs[k]->Cv);
-    const unsigned T = std::max(64u, next_pow2((unsigned long long)b->gs_K * cv + 1ull));
+    unsigned B = 0;
+    unsigned long long most = 0;
+    for (int k = 0; k < b->gs_K; ++k) {
+        const unsigned long long Bk = b->runs[k]->B;
+        unsigned long long n = b->runs[k]->Cv;
+        for (int j = 0; j < k; ++j)
+            n += (b->runs[j]->Cv * std::max<unsigned long long>(Bk, b->runs[j]->B) + Bk - 1) / Bk;
+        most = std::max(most, n);
+        B = std::max(B, b->runs[k]->B);
+    }
+    const unsigned T = std::max(64u, next_pow2(most + 1));
     const size_t slot = b->ks->gs_slot_bytes;
     if ((size_t)T * slot > 200u * 1024u) return FQ_ERR_INVALID;  // segments too large
     int wpb = 4;
     while (wpb > 1 && (size_t)wpb * T * slot > 200u * 1024u) wpb >>= 1;
     CK(b->ks->prepare_gs((size_t)wpb * T * slot));
-    const unsigned B = b->runs[0]->B;
     b->gs_wpb = wpb;
     b->gs_grid = (int)std::max<unsigned long long>(
         1, std::min<unsigned long long>(
@@ -1206,7 +1217,6 @@ static int gs_build(fq_batch* b) {
     GsDesc g;
     memset(&g, 0, sizeof g);
     g.K = b->gs_K;
-    g.B = B;
     g.table = T;
     g.part = b->gs_part;
     g.alpha = b->gs_alpha;
@@ -2048,7 +2058,7 @@ extern "C" int fq_batch_set_overlaps(fq_batch* b, const int* g2_d, int n_g2) {
     if (R < 2 || R > FQ_MAX_REPLICAS) return FQ_ERR_INVALID;
     const fq_run* r0 = b->runs[0];
     for (const fq_run* r : b->runs)
-        if (r->B != r0->B || r->ham.mp.kind != r0->ham.mp.kind || r->ham.mp.M != r0->ham.mp.M ||
+        if (r->size_class != r0->size_class || r->ham.mp.kind != r0->ham.mp.kind || r->ham.mp.M != r0->ham.mp.M ||
             r->ham.mp.N != r0->ham.mp.N || r->ham.mp.Lx != r0->ham.mp.Lx)
             return FQ_ERR_INVALID;
     if (n_g2 && r0->ham.mp.kind != FQ_BH_REAL_1D) return FQ_ERR_INVALID;
@@ -2080,7 +2090,7 @@ extern "C" int fq_batch_set_spectral(fq_batch* b, int K) {
         const fq_run* r0 = b->runs[0];
         for (int k = 0; k < K; ++k) {
             const fq_run* r = b->runs[k];
-            if (r->B != r0->B || r->amp == FQ_AMP_INT || r->ham.mp.M != r0->ham.mp.M ||
+            if (r->size_class != r0->size_class || r->amp == FQ_AMP_INT || r->ham.mp.M != r0->ham.mp.M ||
                 r->ham.mp.N != r0->ham.mp.N || r->ham.mp.kind != r0->ham.mp.kind ||
                 r->ham.mp.Lx != r0->ham.mp.Lx)
                 return FQ_ERR_INVALID;

@@ -1501,8 +1501,9 @@ __global__ void __launch_bounds__(BLOCK) k_shift(const RunDesc* __restrict__ run
 
 // ---------------------------------------------------------------------------
 // replica overlaps (Sec. 4.3, Eq. RayleighQuotientReplica): for every pair
-// (A, B) of a batch's runs and every segment, A's entries go into the warp's
-// on-chip table and B's entries look up theirs; the products c_A,j c_B,j and
+// (A, B) of a batch's runs and every segment of A, A's entries go into the
+// warp's on-chip table and the entries of B's segments of the same addresses
+// look up theirs; the products c_A,j c_B,j and
 // G2(d)_jj c_A,j c_B,j (Eq. g2) are summed per warp.  Each warp writes its
 // own partial sums (no atomics) and k_overlap_row adds them in a fixed order,
 // so the result does not depend on timing.
@@ -1538,8 +1539,7 @@ __global__ void __launch_bounds__(128) k_overlap(const RunDesc* __restrict__ run
     double* const part = od->part + (size_t)gw * P * W;
     for (int i = lane; i < P * W; i += 32) part[i] = 0.0;
     __syncwarp();
-    const unsigned B = od->B;
-    const unsigned long long total = (unsigned long long)P * B;
+    const unsigned long long total = od->first[P];
     const unsigned long long i0 = total * gw / nw, i1 = total * (gw + 1) / nw;
     double acc[1 + FQ_MAX_G2];
     for (int q = 0; q < W; ++q) acc[q] = 0.0;
@@ -1547,6 +1547,7 @@ __global__ void __launch_bounds__(128) k_overlap(const RunDesc* __restrict__ run
     int cur_p = -1;
     const RunDesc *RA = nullptr, *RB = nullptr;
     int ca = 0, cb = 0;
+    unsigned seg = 0, nsa = 0, nsb = 0;  // segment of A; segments of A and B
     auto flush = [&]() {
         for (int q = 0; q < W; ++q) {
             const double v = warp_sum(acc[q]);
@@ -1554,29 +1555,30 @@ __global__ void __launch_bounds__(128) k_overlap(const RunDesc* __restrict__ run
             acc[q] = 0.0;
         }
     };
-    for (unsigned long long it = i0; it < i1; ++it) {
-        const int p = (int)(it / B);
-        const unsigned seg = (unsigned)(it % B);
-        if (p != cur_p) {  // warp-uniform
+    for (unsigned long long it = i0; it < i1; ++it, ++seg) {
+        if (seg == nsa) {  // the first item, or the next pair (warp-uniform)
             if (cur_p >= 0) flush();
-            cur_p = p;
-            RA = runs + od->pa[p];
-            RB = runs + od->pb[p];
+            ++cur_p;
+            while (od->first[cur_p + 1] <= it) ++cur_p;
+            seg = (unsigned)(it - od->first[cur_p]);
+            RA = runs + od->pa[cur_p];
+            RB = runs + od->pb[cur_p];
             ca = RA->st->cur;
             cb = RB->st->cur;
+            nsa = RA->B;
+            nsb = RB->B;
         }
+        unsigned b0, b1;
+        segment_span(seg, nsa, nsb, b0, b1);
         const unsigned na = min(RA->vcount[ca][seg], RA->Cv);
-        const unsigned nb = min(RB->vcount[cb][seg], RB->Cv);
-        // the next segment of the pair into L2 while this one is joined
-        if (lane == 0 && it + 1 < i1 && seg + 1 < B) {
-            prefetch_segment<K, A>(RA, ca, seg + 1);
-            prefetch_segment<K, A>(RB, cb, seg + 1);
+        // the next segments of the pair into L2 while these are joined
+        if (lane == 0 && it + 1 < i1) {
+            if (seg + 1 < nsa) prefetch_segment<K, A>(RA, ca, seg + 1);
+            if (b1 + 1 < nsb) prefetch_segment<K, A>(RB, cb, b1 + 1);
         }
-        if (!na || !nb) continue;
+        if (!na || (b0 == b1 && !RB->vcount[cb][b0])) continue;
         const K* ka = (const K*)RA->vkeys[ca] + (size_t)seg * RA->Cv;
         const A* aa = (const A*)RA->vamps[ca] + (size_t)seg * RA->Cv;
-        const K* kb = (const K*)RB->vkeys[cb] + (size_t)seg * RB->Cv;
-        const A* ab = (const A*)RB->vamps[cb] + (size_t)seg * RB->Cv;
         // A's entries (distinct addresses; the table has more slots than a
         // segment's capacity, so an insert always finds one)
         unsigned nl = 0;
@@ -1593,25 +1595,30 @@ __global__ void __launch_bounds__(128) k_overlap(const RunDesc* __restrict__ run
             nl += __popc(bal);
         }
         __syncwarp();
-        for (unsigned j0 = 0; j0 < nb; j0 += 32) {
-            const unsigned j = j0 + lane;
-            if (j < nb) {
-                const K key = kb[j];
-                const int q = table_find(tk, T - 1u, key);
-                if (q >= 0) {
-                    const double prod = ta[q] * (double)ab[j];
-                    acc[0] += prod;
-                    if (nq) {
-                        const int M = RA->mp.M;
-                        occupations(key, M, occ);
-                        for (int k = 0; k < nq; ++k) {
-                            const int d = od->d[k];
-                            long long sn = 0;
-                            for (int i = 0; i < M; ++i) {
-                                const int i2 = i + d < M ? i + d : i + d - M;
-                                sn += (long long)occ[i] * ((long long)occ[i2] - (d == 0 ? 1 : 0));
+        for (unsigned sb = b0; sb <= b1; ++sb) {
+            const unsigned nb = min(RB->vcount[cb][sb], RB->Cv);
+            const K* kb = (const K*)RB->vkeys[cb] + (size_t)sb * RB->Cv;
+            const A* ab = (const A*)RB->vamps[cb] + (size_t)sb * RB->Cv;
+            for (unsigned j0 = 0; j0 < nb; j0 += 32) {
+                const unsigned j = j0 + lane;
+                if (j < nb) {
+                    const K key = kb[j];
+                    const int q = table_find(tk, T - 1u, key);
+                    if (q >= 0) {
+                        const double prod = ta[q] * (double)ab[j];
+                        acc[0] += prod;
+                        if (nq) {
+                            const int M = RA->mp.M;
+                            occupations(key, M, occ);
+                            for (int k = 0; k < nq; ++k) {
+                                const int d = od->d[k];
+                                long long sn = 0;
+                                for (int i = 0; i < M; ++i) {
+                                    const int i2 = i + d < M ? i + d : i + d - M;
+                                    sn += (long long)occ[i] * ((long long)occ[i2] - (d == 0 ? 1 : 0));
+                                }
+                                acc[1 + k] += ((double)sn / (double)M) * prod;
                             }
-                            acc[1 + k] += ((double)sn / (double)M) * prod;
                         }
                     }
                 }
@@ -1700,12 +1707,14 @@ __global__ void __launch_bounds__(128) k_gs_dots(const RunDesc* __restrict__ run
     for (int i = 0; i < 2 * k; ++i) acc[i] = 0.0;
     const RunDesc* Rk = runs + k;
     const int ck = Rk->st->cur ^ 1;
+    const unsigned nsk = Rk->B;
     unsigned g0, g1;
-    warp_range(gs->B, gw, nw, g0, g1);
+    warp_range(nsk, gw, nw, g0, g1);
     for (unsigned seg = g0; seg < g1; ++seg) {
         if (lane == 0 && seg + 1 < g1) {  // the next segment of every state into L2
             prefetch_segment<K, A>(Rk, ck, seg + 1);
-            for (int j = 0; j < k; ++j) prefetch_segment<K, A>(runs + j, runs[j].st->cur ^ 1, seg + 1);
+            for (int j = 0; j < k; ++j)
+                if (runs[j].B == nsk) prefetch_segment<K, A>(runs + j, runs[j].st->cur ^ 1, seg + 1);
         }
         const unsigned nk = min(Rk->vcount[ck][seg], Rk->Cv);
         const K* kk = (const K*)Rk->vkeys[ck] + (size_t)seg * Rk->Cv;
@@ -1727,15 +1736,22 @@ __global__ void __launch_bounds__(128) k_gs_dots(const RunDesc* __restrict__ run
         for (int j = 0; j < k; ++j) {
             const RunDesc* Rj = runs + j;
             const int cj = Rj->st->cur ^ 1;
-            const unsigned nj = min(Rj->vcount[cj][seg], Rj->Cv);
-            const K* jk = (const K*)Rj->vkeys[cj] + (size_t)seg * Rj->Cv;
-            const A* ja = (const A*)Rj->vamps[cj] + (size_t)seg * Rj->Cv;
-            for (unsigned i = lane; i < nj; i += 32) {
-                const double v = (double)ja[i];
-                acc[2 * j + 1] += v * v;
-                if (nk) {
-                    const int q = table_find(tk, T - 1u, jk[i]);
-                    if (q >= 0) acc[2 * j] += v * ta[q];
+            const unsigned nsj = Rj->B;
+            unsigned b0, b1;
+            segment_span(seg, nsk, nsj, b0, b1);
+            for (unsigned sj = b0; sj <= b1; ++sj) {
+                const unsigned nj = min(Rj->vcount[cj][sj], Rj->Cv);
+                const K* jk = (const K*)Rj->vkeys[cj] + (size_t)sj * Rj->Cv;
+                const A* ja = (const A*)Rj->vamps[cj] + (size_t)sj * Rj->Cv;
+                for (unsigned i = lane; i < nj; i += 32) {
+                    // an entry counts where its address lies in run k's map
+                    if (nsj != nsk && segment_of(seg_hash(jk[i]), nsk) != seg) continue;
+                    const double v = (double)ja[i];
+                    acc[2 * j + 1] += v * v;
+                    if (nk) {
+                        const int q = table_find(tk, T - 1u, jk[i]);
+                        if (q >= 0) acc[2 * j] += v * ta[q];
+                    }
                 }
             }
         }
@@ -1804,11 +1820,13 @@ __global__ void __launch_bounds__(128) k_gs_axpy(const RunDesc* __restrict__ run
     for (int j = 0; j < k; ++j) alpha[j] = gs->alpha[j];
     MergeAcc acc;
     unsigned g0, g1;
-    warp_range(gs->B, gw, nw, g0, g1);
+    const unsigned nsk = R->B;
+    warp_range(nsk, gw, nw, g0, g1);
     for (unsigned seg = g0; seg < g1; ++seg) {
         if (lane == 0 && seg + 1 < g1) {  // the next segment of every state into L2
             prefetch_segment<K, A>(R, ck, seg + 1);
-            for (int j = 0; j < k; ++j) prefetch_segment<K, A>(runs + j, runs[j].st->cur ^ 1, seg + 1);
+            for (int j = 0; j < k; ++j)
+                if (runs[j].B == nsk) prefetch_segment<K, A>(runs + j, runs[j].st->cur ^ 1, seg + 1);
         }
         const unsigned nk = min(R->vcount[ck][seg], Cv);
         K* const kk = (K*)R->vkeys[ck] + (size_t)seg * Cv;
@@ -1818,31 +1836,37 @@ __global__ void __launch_bounds__(128) k_gs_axpy(const RunDesc* __restrict__ run
         for (int j = -1; j < k; ++j) {
             const RunDesc* Rj = j < 0 ? R : runs + j;
             const int cj = j < 0 ? ck : (Rj->st->cur ^ 1);
-            const unsigned nj = j < 0 ? nk : min(Rj->vcount[cj][seg], Rj->Cv);
-            const K* jk = (const K*)Rj->vkeys[cj] + (size_t)seg * Rj->Cv;
-            const A* ja = (const A*)Rj->vamps[cj] + (size_t)seg * Rj->Cv;
-            for (unsigned i0 = 0; i0 < nj; i0 += 32) {
-                const unsigned i = i0 + lane;
-                bool is_new = false;
-                int q = -1;
-                if (i < nj) {
-                    q = table_insert(tk, T - 1u, jk[i], is_new);
-                    if (q < 0) {
-                        acc.full = true;
-                    } else if (j < 0) {
-                        ta[q] = (ACC)ja[i];
-                    } else {
-                        const ACC v = is_new ? (ACC)0 : ta[q];
-                        if constexpr (AMP == FQ_AMP_F32)
-                            ta[q] = v - (float)alpha[j] * ja[i];
-                        else
-                            ta[q] = v - (ACC)(alpha[j] * (double)ja[i]);
-                        tc[q] = 1;
+            const unsigned nsj = Rj->B;
+            unsigned b0, b1;
+            segment_span(seg, nsk, nsj, b0, b1);
+            for (unsigned sj = b0; sj <= b1; ++sj) {
+                const unsigned nj = j < 0 ? nk : min(Rj->vcount[cj][sj], Rj->Cv);
+                const K* jk = (const K*)Rj->vkeys[cj] + (size_t)sj * Rj->Cv;
+                const A* ja = (const A*)Rj->vamps[cj] + (size_t)sj * Rj->Cv;
+                for (unsigned i0 = 0; i0 < nj; i0 += 32) {
+                    const unsigned i = i0 + lane;
+                    bool is_new = false;
+                    int q = -1;
+                    // entries whose address lies in run k's segment
+                    if (i < nj && (nsj == nsk || segment_of(seg_hash(jk[i]), nsk) == seg)) {
+                        q = table_insert(tk, T - 1u, jk[i], is_new);
+                        if (q < 0) {
+                            acc.full = true;
+                        } else if (j < 0) {
+                            ta[q] = (ACC)ja[i];
+                        } else {
+                            const ACC v = is_new ? (ACC)0 : ta[q];
+                            if constexpr (AMP == FQ_AMP_F32)
+                                ta[q] = v - (float)alpha[j] * ja[i];
+                            else
+                                ta[q] = v - (ACC)(alpha[j] * (double)ja[i]);
+                            tc[q] = 1;
+                        }
                     }
+                    const unsigned bal = __ballot_sync(0xFFFFFFFFu, is_new);
+                    if (is_new) tl[nl + __popc(bal & ((1u << lane) - 1u))] = (unsigned)q;
+                    nl += __popc(bal);
                 }
-                const unsigned bal = __ballot_sync(0xFFFFFFFFu, is_new);
-                if (is_new) tl[nl + __popc(bal & ((1u << lane) - 1u))] = (unsigned)q;
-                nl += __popc(bal);
             }
             __syncwarp();
         }

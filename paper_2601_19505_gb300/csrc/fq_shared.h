@@ -30,7 +30,26 @@
 #define FQ_MAX_MOM_MODES 64
 #define FQ_HIST_CAP 65536u
 
+#ifdef __CUDACC__
+#define FQ_HOST_DEVICE __host__ __device__ __forceinline__
+#else
+#define FQ_HOST_DEVICE inline
+#endif
+
 namespace fq {
+
+// The segments [lo, hi] of a run with `there` segments that can hold an
+// address of segment `seg` of a run with `here`: segment_of scales the hash's
+// high word, so a segment is a range of it.
+FQ_HOST_DEVICE void segment_span(unsigned seg, unsigned here, unsigned there, unsigned& lo,
+                                 unsigned& hi) {
+    lo = hi = seg;
+    if (here == there) return;
+    const unsigned long long first = (((unsigned long long)seg << 32) + here - 1) / here;
+    const unsigned long long end = ((((unsigned long long)seg + 1) << 32) + here - 1) / here;
+    lo = (unsigned)((first * there) >> 32);
+    hi = (unsigned)(((end - 1) * there) >> 32);
+}
 
 struct ModelParams {
     int kind, M, N, Lx, Ly, nbits;
@@ -119,17 +138,17 @@ struct RunDesc {
 };
 
 // Replica overlaps of a batch (Sec. 4.3): for every pair (A, B) of its runs,
-// c_A^T c_B and c_A^T G2(d_k) c_B (Eq. g2) after each step.  The runs share
-// one segment map (equal B), so segment b of A and of B hold the same
-// addresses' entries.
+// c_A^T c_B and c_A^T G2(d_k) c_B (Eq. g2) after each step.  The addresses of
+// a segment of A lie in one or a few segments of B (segment_span; in the same
+// one when the runs have equally many).
 #define FQ_MAX_REPLICAS 8
+#define FQ_MAX_PAIRS (FQ_MAX_REPLICAS * (FQ_MAX_REPLICAS - 1) / 2)
 #define FQ_MAX_G2 16
 struct OverlapDesc {
     int R, P, nq;                  // runs, pairs, G2 distances
     int d[FQ_MAX_G2];
-    int pa[FQ_MAX_REPLICAS * (FQ_MAX_REPLICAS - 1) / 2];
-    int pb[FQ_MAX_REPLICAS * (FQ_MAX_REPLICAS - 1) / 2];
-    unsigned B;                    // segments per run
+    int pa[FQ_MAX_PAIRS], pb[FQ_MAX_PAIRS];
+    unsigned long long first[FQ_MAX_PAIRS + 1];  // pair p's first item: one per segment of A
     unsigned table;                // slots of a warp's table (power of 2)
     double* part;                  // per warp: P x (1 + nq) partial sums
     double* ring;                  // rows of width 1 + P (1 + nq)
@@ -143,7 +162,6 @@ struct OverlapDesc {
 #define FQ_MAX_SPECTRAL 8
 struct GsDesc {
     int K;                  // spectral states
-    unsigned B;             // segments per run
     unsigned table;         // slots of a warp's table (power of 2)
     double* part;           // per warp: 2 FQ_MAX_SPECTRAL partial dot products
     double* alpha;          // FQ_MAX_SPECTRAL coefficients of the run being orthogonalised
