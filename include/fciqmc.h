@@ -104,7 +104,12 @@ enum {
  * annihilation: FQ_ANN_*.  seed, run_id: key of the counter-based random
  * draws.  compression: FQ_COMPRESS_*.  capacity_vec, capacity_spawn: maximum
  * occupied entries of the vector and spawn entries per step (0 = derived from
- * target and threshold). */
+ * target and threshold).  Both are kept in hash segments with room for the
+ * segments' fluctuations.  Spawns arrive in clumps of one address, and the
+ * small buckets of runs below about 4e5 walkers have a full bucket's room
+ * each, so that their spawn buffers are up to 5.3 times as large (derived
+ * capacities, 64-bit addresses, FP64: spawn buffers of 4.8 MB at 1e4 walkers,
+ * 30 MB at 1e5, 86 MB at 1e6; vectors of 1.4, 12.5 and 90 MB). */
 typedef struct {
     double dt, target, zeta, xi, threshold, t_rel;
     int32_t mode, annihilation;
@@ -259,7 +264,9 @@ int fq_run_spawns(fq_run *r, fq_key *dest, double *val, size_t cap, size_t *n);
  * at their old size; should even that fail, every later step and check of
  * the run returns FQ_ERR_NOMEM).  Synchronises. */
 int fq_run_reserve(fq_run *r, size_t capacity_vec, size_t capacity_spawn);
-/* Current total capacities (entries of the vector, spawns per step). */
+/* Current total capacities (entries of the vector, spawns per step).  They
+ * are the numbers that fq_run_reserve takes: reserving more than them grows
+ * the run. */
 int fq_run_capacity(const fq_run *r, size_t *capacity_vec, size_t *capacity_spawn);
 /* Annihilation tables (tests and tuning; not in the paper).  A bucket's
  * spawns are summed in an on-chip table of `slots` entries per merge warp

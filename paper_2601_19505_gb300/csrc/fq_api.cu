@@ -22,6 +22,7 @@
 #include "fq_launch.h"
 #include "fq_shared.h"
 #include "fq_shares.h"
+#include "fq_sizes.h"
 
 using namespace fq;
 
@@ -92,6 +93,7 @@ struct fq_run {
     unsigned B, Cv, Cs, slots;  // slots: on-chip table slots per merge warp
     unsigned Cp;                // spawn slots per bucket in the dense primary region
     unsigned size_class;        // full buckets, rounded up to a power of two (joinable)
+    SpawnRoom room;             // the buckets' spawn slots for a capacity
     double fill;                // steady-state spawns per bucket
     bool no_spawn_buf;          // a failed growth left no spawn buffers: the run cannot step
     RunState* st;
@@ -213,12 +215,6 @@ static void dev_free_all(fq_run* r) {
         else cudaFreeAsync(a.p, r->stream);
     }
     r->allocs.clear();
-}
-
-static unsigned next_pow2(unsigned long long x) {
-    unsigned p = 1;
-    while (p < x) p <<= 1;
-    return p;
 }
 
 static int num_sms() {
@@ -617,46 +613,6 @@ static void table_sizes(fq_run* r) {
         32768, next_pow2((unsigned long long)r->Cv + r->Cs));
 }
 
-// segments whose buckets fill a third of a merge warp's table of `slots`
-static double full_segments(double s_ss, unsigned slots) {
-    return std::max(1.0, std::ceil(std::min(s_ss / (slots / 3.0), 268000000.0)));
-}
-
-// Segments for s_ss spawns a step.  Large runs: full buckets, and a multiple
-// of the warps that are resident at once (16 per SM in the default launch
-// shape), so that every warp takes the same number: with a power of two, 1e6
-// walkers were 8192 buckets on 2432 warps, where some took four and most
-// three (now 7296: 8 % off the step), and 1e8 walkers 2^20 of 105 spawns
-// instead of 646912 of 170 (2 %).  Below one full bucket per warp, smaller
-// buckets on more warps, down to one round of 32 spawns: a step of 1e4
-// walkers on 12 sites took 39 us with buckets of 86 spawns and takes 33 with
-// 32, 1e5 on 20 sites 42 and 37.  Less than 64 such buckets (2000 walkers, in
-// spaces where a few addresses draw most of the spawns) stay at 100.
-static unsigned segments_for(double s_ss, unsigned slots) {
-    const double warps = num_sms() * 16.0, full = full_segments(s_ss, slots);
-    if (full > warps) return (unsigned)(std::ceil(full / warps) * warps);
-    const double fine = std::ceil(s_ss / (s_ss < 64.0 * 32.0 ? 100.0 : 32.0));
-    return (unsigned)std::max(1.0, std::min(warps, fine));
-}
-
-// per-segment capacities for totals lcap, scap over B segments (spawns
-// arrive in clumps of up to k, see fq_run_create)
-static void segment_caps(double lcap, double scap, unsigned B, double k, unsigned& Cv, unsigned& Cs) {
-    const double mv = lcap / B, ms = scap / B;
-    Cv = (unsigned)((mv + 4.0 * std::sqrt(mv) + 16.0 + 31.0) / 32.0) * 32u;
-    Cs = (unsigned)((ms + 4.0 * std::sqrt(ms * k) + k + 16.0 + 31.0) / 32.0) * 32u;
-}
-
-// Spawn slots per bucket in the dense primary region: the steady-state fill
-// plus three standard deviations of its compound-Poisson count (a multiple
-// of 32, at most the bucket's capacity), so that nearly every spawn of an
-// equilibrated run is stored there.
-static unsigned primary_slots(double s_ss, unsigned B, double k, unsigned Cs) {
-    const double m = s_ss / B;
-    const unsigned p = (unsigned)((m + 3.0 * std::sqrt(m * k) + 16.0 + 31.0) / 32.0) * 32u;
-    return std::min(p, Cs);
-}
-
 static void batch_free(fq_batch* b);
 static int batch_build(fq_batch* b);
 
@@ -696,13 +652,16 @@ extern "C" int fq_run_create(fq_run** out, const fq_ham* h, const fq_params* p, 
     const double th = r->det ? 1.0 : (p->mode == FQ_MODE_INT ? 1.0 : std::min(1.0, p->threshold));
     // the spawn count follows the norm, not the occupied count: when the
     // vector fills a small Hilbert space its entries grow and spawn more
-    const double lnorm = p->capacity_vec ? (double)p->capacity_vec : 2.0 * p->target / th + 1024.0;
-    double lcap = lnorm;
-    if (r->det && !p->capacity_vec) lcap = std::min(dim * 1.05 + 1024.0, 1.0e9);
-    lcap = std::min(lcap, dim * 1.05 + 1024.0);
-    double scap = p->capacity_spawn ? (double)p->capacity_spawn
-                                    : 1.5 * lnorm * std::max(1.0, p->t_rel) + 4096.0;
-    if (r->det && !p->capacity_spawn) scap = lcap * (double)max_offdiag(h->mp) + 4096.0;
+    const double all = dim * 1.05 + 1024.0;  // every address of a small space
+    auto vec_cap = [&](double norm) { return std::min(norm, all); };
+    auto spawn_cap = [&](double norm, double len) {
+        return r->det ? len * (double)max_offdiag(h->mp) + 4096.0
+                      : 1.5 * norm * std::max(1.0, p->t_rel) + 4096.0;
+    };
+    const double usual_norm = r->det ? 1.0e9 : 2.0 * p->target / th + 1024.0;
+    const double lnorm = p->capacity_vec ? (double)p->capacity_vec : usual_norm;
+    const double lcap = vec_cap(lnorm);
+    const double scap = p->capacity_spawn ? (double)p->capacity_spawn : spawn_cap(lnorm, lcap);
     if (lcap > 4.0e9 || scap > 8.0e9) {
         delete r;
         return FQ_ERR_INVALID;
@@ -716,19 +675,16 @@ extern "C" int fq_run_create(fq_run** out, const fq_ham* h, const fq_params* p, 
         l_ss = std::min(lcap, dim);
         s_ss = l_ss * (double)max_offdiag(h->mp);
     }
-    r->B = segments_for(s_ss, r->slots);
+    r->B = segments_for(s_ss, r->slots, num_sms());
     r->size_class = next_pow2((unsigned long long)full_segments(s_ss, r->slots));
     {
         // spawns arrive in clumps (one address receives spawns from many
         // sources; every neighbour's in the deterministic limit), so the
         // bucket count fluctuates like a compound Poisson sum with clump size k
         const double k = r->det ? (double)max_offdiag(h->mp) : 8.0;
-        unsigned c = 0;
-        segment_caps(lcap, scap, r->B, k, r->Cv, r->Cs);
-        // spawns come in clumps of one address, which a small bucket feels
-        // more: it has the room of a full one
-        segment_caps(lcap, scap, (unsigned)std::min<double>(r->B, full_segments(s_ss, r->slots)), k,
-                     c, r->Cs);
+        r->room = spawn_room(r->B, full_segments(s_ss, r->slots), k, spawn_cap(usual_norm, lcap));
+        r->Cv = vec_slots(lcap, r->B);
+        r->Cs = r->room.slots(scap);
         r->Cp = primary_slots(s_ss, r->B, k, r->Cs);
         r->fill = std::min(s_ss / r->B, 1e6);
         table_sizes(r);
@@ -1629,11 +1585,8 @@ extern "C" int fq_run_reserve(fq_run* r, size_t capacity_vec, size_t capacity_sp
     if (!r) return FQ_ERR_INVALID;
     int rc = run_check(r);
     if (rc) return rc;
-    const double k = r->det ? (double)max_offdiag(r->ham.mp) : 8.0;
-    unsigned Cv, Cs;
-    segment_caps((double)capacity_vec, (double)capacity_spawn, r->B, k, Cv, Cs);
-    Cv = std::max(Cv, r->Cv);
-    Cs = std::max(Cs, r->Cs);
+    const unsigned Cv = std::max(vec_slots((double)capacity_vec, r->B), r->Cv);
+    const unsigned Cs = std::max(r->room.slots((double)capacity_spawn), r->Cs);
     if (Cv == r->Cv && Cs == r->Cs) return FQ_OK;
     const size_t kb = r->ks->key_bytes, ab = r->ks->amp_bytes, sb = r->ks->spawn_bytes;
     int cur = 0;
@@ -1694,7 +1647,7 @@ extern "C" int fq_run_reserve(fq_run* r, size_t capacity_vec, size_t capacity_sp
 extern "C" int fq_run_capacity(const fq_run* r, size_t* capacity_vec, size_t* capacity_spawn) {
     if (!r) return FQ_ERR_INVALID;
     if (capacity_vec) *capacity_vec = (size_t)r->B * r->Cv;
-    if (capacity_spawn) *capacity_spawn = (size_t)r->B * r->Cs;
+    if (capacity_spawn) *capacity_spawn = (size_t)r->room.total(r->Cs);
     return FQ_OK;
 }
 
