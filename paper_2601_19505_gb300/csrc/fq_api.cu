@@ -159,8 +159,9 @@ struct fq_batch {
     size_t ov_part_n;
     double* ov_ring;
     unsigned long long* ov_head;
-    unsigned ov_cap, ov_table;
-    int ov_grid, ov_wpb;
+    unsigned ov_cap;
+    JoinShape ov_shape;
+    unsigned char* ov_tables;    // device-memory tables of a join of large segments
     unsigned long long ov_read;  // rows handed out so far
     // excited states (fq_batch_set_spectral)
     int gs_K;
@@ -168,8 +169,8 @@ struct fq_batch {
     double* gs_part;
     double* gs_alpha;
     size_t gs_part_n;
-    unsigned gs_table;
-    int gs_grid, gs_wpb;
+    JoinShape gs_shape;
+    unsigned char* gs_tables;
 };
 
 // ---------------------------------------------------------------------------
@@ -1023,13 +1024,13 @@ extern "C" int fq_run_set_target(fq_run* r, double t) {
 // batches: descriptor table, graphs, stepping
 
 static void launch_overlaps(fq_batch* b, cudaStream_t s) {
-    if (b->ov_on) b->ks->overlap(b->d_desc, b->d_ov, b->ov_grid, b->ov_wpb, b->ov_table, s);
+    if (b->ov_on) b->ks->overlap(b->d_desc, b->d_ov, b->ov_shape, s);
 }
 
 // Gram-Schmidt of the spectral states, between the merge and the shift update
 static void launch_gs(fq_batch* b, cudaStream_t s) {
     for (int k = 1; k < b->gs_K; ++k)
-        b->ks->gs(b->d_desc, b->d_gs, k, b->gs_grid, b->gs_wpb, b->gs_table, s);
+        b->ks->gs(b->d_desc, b->d_gs, k, b->gs_shape, s);
 }
 
 static void enqueue_steps(fq_batch* b, int n, cudaStream_t s) {
@@ -1058,19 +1059,49 @@ static void batch_release(fq_batch* b) {
 static void overlaps_free(fq_batch* b) {
     if (b->d_ov) cudaFree(b->d_ov);
     if (b->ov_part) cudaFree(b->ov_part);
+    if (b->ov_tables) cudaFree(b->ov_tables);
     if (b->ov_ring) cudaFree(b->ov_ring);
     if (b->ov_head) cudaFree(b->ov_head);
     b->d_ov = nullptr;
     b->ov_part = b->ov_ring = nullptr;
+    b->ov_tables = nullptr;
     b->ov_head = nullptr;
     b->ov_part_n = 0;
     b->ov_on = false;
 }
 
-// blocks per SM for a join kernel with `smem` bytes of tables per block:
-// as many as the SM's 228 KB hold (1 KB of it reserved per block), at most 8
-static unsigned long long join_blocks_per_sm(size_t smem) {
-    return std::max<size_t>(1, std::min<size_t>(8, (228u * 1024u) / (smem + 1024u)));
+// The most on-chip memory of a block of a join.  The kernels are allowed this
+// much whatever a batch needs: the allowance is the function's, and a smaller
+// batch's would make an earlier one's launches fail.
+constexpr size_t kJoinSmem = 200u * 1024u;
+
+// The launch of a join of `items` segments with tables of T slots: on-chip
+// tables of up to four warps a block, and as many blocks as the SM's 228 KB
+// hold (1 KB of it reserved per block), at most 8 an SM.  A table beyond 200 KB
+// lies in device memory, four warps an SM (`tables`, allocated anew; up to
+// 800 KB each): segments of a capacity some times the derived one, which
+// segment counts that are powers of two kept below 200 KB or not.
+static int join_shape(size_t slot, unsigned T, unsigned long long items, JoinShape& j,
+                      unsigned char*& tables) {
+    const size_t one = (size_t)T * slot;
+    if (tables) cudaFree(tables);
+    tables = nullptr;
+    if (one > 4 * kJoinSmem) return FQ_ERR_INVALID;  // segments too large
+    j.table = T;
+    j.dev = j.any = one > kJoinSmem;
+    j.wpb = 4;
+    while (!j.dev && j.wpb > 1 && j.wpb * one > kJoinSmem) j.wpb >>= 1;
+    const unsigned long long per_sm =
+        j.dev ? 1 : std::max<size_t>(1, std::min<size_t>(8, (228u * 1024u) / (j.wpb * one + 1024u)));
+    j.grid = (int)std::max<unsigned long long>(
+        1, std::min<unsigned long long>((unsigned long long)num_sms() * per_sm,
+                                        (items + j.wpb - 1) / j.wpb));
+    if (j.dev && cudaMalloc((void**)&tables, (size_t)j.grid * j.wpb * one) != cudaSuccess) {
+        cudaGetLastError();
+        tables = nullptr;
+        return FQ_ERR_NOMEM;
+    }
+    return FQ_OK;
 }
 
 // the overlap launch for the batch's current sizes: one table per warp with
@@ -1081,12 +1112,6 @@ static int overlaps_build(fq_batch* b) {
     unsigned cv = 0;
     for (fq_run* r : b->runs) cv = std::max(cv, r->Cv);
     const unsigned T = std::max(64u, next_pow2(cv + 1ull));
-    const size_t slot = b->ks->overlap_slot_bytes;
-    int wpb = 4;
-    while (wpb > 1 && (size_t)wpb * T * slot > 200u * 1024u) wpb >>= 1;
-    if ((size_t)T * slot > 200u * 1024u) return FQ_ERR_INVALID;  // segments too large
-    const size_t smem = (size_t)wpb * T * slot;
-    CK(b->ks->prepare_overlap(smem));
     const int R = (int)b->runs.size(), P = R * (R - 1) / 2;
     OverlapDesc od;
     memset(&od, 0, sizeof od);
@@ -1097,13 +1122,12 @@ static int overlaps_build(fq_batch* b) {
             od.pb[p] = c;
             od.first[p + 1] = od.first[p] + b->runs[a]->B;
         }
-    const unsigned long long items = od.first[P];
-    b->ov_wpb = wpb;
-    b->ov_grid = (int)std::max<unsigned long long>(
-        1, std::min<unsigned long long>((unsigned long long)num_sms() * join_blocks_per_sm(smem),
-                                        (items + wpb - 1) / wpb));
-    b->ov_table = T;
-    const size_t need = (size_t)b->ov_grid * wpb * P * (1 + b->ov_nq);
+    JoinShape& j = b->ov_shape;
+    const int rc = join_shape(b->ks->overlap_slot_bytes, T, od.first[P], j, b->ov_tables);
+    if (rc) return rc;
+    for (const fq_run* r : b->runs) j.any |= r->B != b->runs[0]->B;
+    CK(b->ks->prepare_overlap(kJoinSmem));
+    const size_t need = (size_t)j.grid * j.wpb * P * (1 + b->ov_nq);
     if (need > b->ov_part_n) {
         if (b->ov_part) cudaFree(b->ov_part);
         b->ov_part = nullptr;
@@ -1116,6 +1140,7 @@ static int overlaps_build(fq_batch* b) {
     od.nq = b->ov_nq;
     for (int k = 0; k < b->ov_nq; ++k) od.d[k] = b->ov_d[k];
     od.table = T;
+    od.tables = b->ov_tables;
     od.part = b->ov_part;
     od.ring = b->ov_ring;
     od.head = b->ov_head;
@@ -1127,9 +1152,11 @@ static int overlaps_build(fq_batch* b) {
 static void gs_free(fq_batch* b) {
     if (b->d_gs) cudaFree(b->d_gs);
     if (b->gs_part) cudaFree(b->gs_part);
+    if (b->gs_tables) cudaFree(b->gs_tables);
     if (b->gs_alpha) cudaFree(b->gs_alpha);
     b->d_gs = nullptr;
     b->gs_part = b->gs_alpha = nullptr;
+    b->gs_tables = nullptr;
     b->gs_part_n = 0;
     b->gs_K = 0;
 }
@@ -1151,18 +1178,12 @@ static int gs_build(fq_batch* b) {
         B = std::max(B, b->runs[k]->B);
     }
     const unsigned T = std::max(64u, next_pow2(most + 1));
-    const size_t slot = b->ks->gs_slot_bytes;
-    if ((size_t)T * slot > 200u * 1024u) return FQ_ERR_INVALID;  // segments too large
-    int wpb = 4;
-    while (wpb > 1 && (size_t)wpb * T * slot > 200u * 1024u) wpb >>= 1;
-    CK(b->ks->prepare_gs((size_t)wpb * T * slot));
-    b->gs_wpb = wpb;
-    b->gs_grid = (int)std::max<unsigned long long>(
-        1, std::min<unsigned long long>(
-               (unsigned long long)num_sms() * join_blocks_per_sm((size_t)wpb * T * slot),
-               ((unsigned long long)B + wpb - 1) / wpb));
-    b->gs_table = T;
-    const size_t need = (size_t)b->gs_grid * wpb * 2 * FQ_MAX_SPECTRAL;
+    JoinShape& j = b->gs_shape;
+    const int rc = join_shape(b->ks->gs_slot_bytes, T, B, j, b->gs_tables);
+    if (rc) return rc;
+    for (int k = 0; k < b->gs_K; ++k) j.any |= b->runs[k]->B != b->runs[0]->B;
+    CK(b->ks->prepare_gs(kJoinSmem));
+    const size_t need = (size_t)j.grid * j.wpb * 2 * FQ_MAX_SPECTRAL;
     if (need > b->gs_part_n) {
         if (b->gs_part) cudaFree(b->gs_part);
         b->gs_part = nullptr;
@@ -1174,6 +1195,7 @@ static int gs_build(fq_batch* b) {
     memset(&g, 0, sizeof g);
     g.K = b->gs_K;
     g.table = T;
+    g.tables = b->gs_tables;
     g.part = b->gs_part;
     g.alpha = b->gs_alpha;
     CK(cudaMemcpy(b->d_gs, &g, sizeof g, cudaMemcpyHostToDevice));

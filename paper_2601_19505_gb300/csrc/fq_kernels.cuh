@@ -1521,14 +1521,20 @@ __device__ __forceinline__ void occupations(K key, int M, unsigned char* occ) {
     }
 }
 
-template <class K, int AMP, int KIND>
-__global__ void __launch_bounds__(128) k_overlap(const RunDesc* __restrict__ runs,
-                                                 const OverlapDesc* __restrict__ od) {
+// ANY: runs of unequal segment counts, or tables in device memory (segments too
+// large for on-chip ones).  A kernel of its own: with the spans and a table
+// anywhere, equal runs joined 1 % slower.
+template <class K, int AMP, int KIND, bool ANY>
+__global__ void __launch_bounds__(128, 8)
+    k_overlap(const RunDesc* __restrict__ runs, const OverlapDesc* __restrict__ od) {
     typedef typename AmpT<AMP>::A A;
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, wpb = blockDim.x >> 5;
     const unsigned T = od->table;
-    unsigned char* base = smem + (size_t)wib * T * (sizeof(K) + sizeof(double) + sizeof(unsigned));
+    const size_t bytes = (size_t)T * (sizeof(K) + sizeof(double) + sizeof(unsigned));
+    unsigned char* base =
+        ANY && od->tables ? od->tables + (size_t)(blockIdx.x * wpb + wib) * bytes
+                          : smem + (size_t)wib * bytes;
     K* const tk = (K*)base;
     double* const ta = (double*)(base + (size_t)T * sizeof(K));
     unsigned* const tl = (unsigned*)(base + (size_t)T * (sizeof(K) + sizeof(double)));
@@ -1568,8 +1574,8 @@ __global__ void __launch_bounds__(128) k_overlap(const RunDesc* __restrict__ run
             nsa = RA->B;
             nsb = RB->B;
         }
-        unsigned b0, b1;
-        segment_span(seg, nsa, nsb, b0, b1);
+        unsigned b0 = seg, b1 = seg;
+        if constexpr (ANY) segment_span(seg, nsa, nsb, b0, b1);
         const unsigned na = min(RA->vcount[ca][seg], RA->Cv);
         // the next segments of the pair into L2 while these are joined
         if (lane == 0 && it + 1 < i1) {
@@ -1688,14 +1694,17 @@ static __global__ void __launch_bounds__(kRowThreads)
 // compresses every changed value by Pi with the draw of stream 0xFFFFFFFC of
 // its address, and rewrites run k's segment in place with its norm terms.
 
-template <class K, int AMP>
+template <class K, int AMP, bool ANY>
 __global__ void __launch_bounds__(128) k_gs_dots(const RunDesc* __restrict__ runs,
                                                  const GsDesc* __restrict__ gs, int k) {
     typedef typename AmpT<AMP>::A A;
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, wpb = blockDim.x >> 5;
     const unsigned T = gs->table;
-    unsigned char* base = smem + (size_t)wib * T * (sizeof(K) + sizeof(double) + sizeof(unsigned));
+    const size_t bytes = (size_t)T * (sizeof(K) + sizeof(double) + sizeof(unsigned));
+    unsigned char* base =
+        ANY && gs->tables ? gs->tables + (size_t)(blockIdx.x * wpb + wib) * bytes
+                          : smem + (size_t)wib * bytes;
     K* const tk = (K*)base;
     double* const ta = (double*)(base + (size_t)T * sizeof(K));
     unsigned* const tl = (unsigned*)(base + (size_t)T * (sizeof(K) + sizeof(double)));
@@ -1714,7 +1723,7 @@ __global__ void __launch_bounds__(128) k_gs_dots(const RunDesc* __restrict__ run
         if (lane == 0 && seg + 1 < g1) {  // the next segment of every state into L2
             prefetch_segment<K, A>(Rk, ck, seg + 1);
             for (int j = 0; j < k; ++j)
-                if (runs[j].B == nsk) prefetch_segment<K, A>(runs + j, runs[j].st->cur ^ 1, seg + 1);
+                if (!ANY || runs[j].B == nsk) prefetch_segment<K, A>(runs + j, runs[j].st->cur ^ 1, seg + 1);
         }
         const unsigned nk = min(Rk->vcount[ck][seg], Rk->Cv);
         const K* kk = (const K*)Rk->vkeys[ck] + (size_t)seg * Rk->Cv;
@@ -1737,15 +1746,15 @@ __global__ void __launch_bounds__(128) k_gs_dots(const RunDesc* __restrict__ run
             const RunDesc* Rj = runs + j;
             const int cj = Rj->st->cur ^ 1;
             const unsigned nsj = Rj->B;
-            unsigned b0, b1;
-            segment_span(seg, nsk, nsj, b0, b1);
+            unsigned b0 = seg, b1 = seg;
+            if constexpr (ANY) segment_span(seg, nsk, nsj, b0, b1);
             for (unsigned sj = b0; sj <= b1; ++sj) {
                 const unsigned nj = min(Rj->vcount[cj][sj], Rj->Cv);
                 const K* jk = (const K*)Rj->vkeys[cj] + (size_t)sj * Rj->Cv;
                 const A* ja = (const A*)Rj->vamps[cj] + (size_t)sj * Rj->Cv;
                 for (unsigned i = lane; i < nj; i += 32) {
                     // an entry counts where its address lies in run k's map
-                    if (nsj != nsk && segment_of(seg_hash(jk[i]), nsk) != seg) continue;
+                    if (ANY && nsj != nsk && segment_of(seg_hash(jk[i]), nsk) != seg) continue;
                     const double v = (double)ja[i];
                     acc[2 * j + 1] += v * v;
                     if (nk) {
@@ -1785,7 +1794,7 @@ static __global__ void __launch_bounds__(kRowThreads)
     }
 }
 
-template <class K, int AMP, int KIND>
+template <class K, int AMP, int KIND, bool ANY>
 __global__ void __launch_bounds__(128) k_gs_axpy(const RunDesc* __restrict__ runs,
                                                  const GsDesc* __restrict__ gs, int k) {
     typedef typename AmpT<AMP>::A A;
@@ -1793,8 +1802,10 @@ __global__ void __launch_bounds__(128) k_gs_axpy(const RunDesc* __restrict__ run
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, wpb = blockDim.x >> 5;
     const unsigned T = gs->table;
+    const size_t bytes = (size_t)T * (sizeof(K) + sizeof(ACC) + sizeof(unsigned) + 1);
     unsigned char* base =
-        smem + (size_t)wib * T * (sizeof(K) + sizeof(ACC) + sizeof(unsigned) + 1);
+        ANY && gs->tables ? gs->tables + (size_t)(blockIdx.x * wpb + wib) * bytes
+                          : smem + (size_t)wib * bytes;
     K* const tk = (K*)base;
     ACC* const ta = (ACC*)(base + (size_t)T * sizeof(K));
     unsigned* const tl = (unsigned*)(base + (size_t)T * (sizeof(K) + sizeof(ACC)));
@@ -1826,7 +1837,7 @@ __global__ void __launch_bounds__(128) k_gs_axpy(const RunDesc* __restrict__ run
         if (lane == 0 && seg + 1 < g1) {  // the next segment of every state into L2
             prefetch_segment<K, A>(R, ck, seg + 1);
             for (int j = 0; j < k; ++j)
-                if (runs[j].B == nsk) prefetch_segment<K, A>(runs + j, runs[j].st->cur ^ 1, seg + 1);
+                if (!ANY || runs[j].B == nsk) prefetch_segment<K, A>(runs + j, runs[j].st->cur ^ 1, seg + 1);
         }
         const unsigned nk = min(R->vcount[ck][seg], Cv);
         K* const kk = (K*)R->vkeys[ck] + (size_t)seg * Cv;
@@ -1837,8 +1848,8 @@ __global__ void __launch_bounds__(128) k_gs_axpy(const RunDesc* __restrict__ run
             const RunDesc* Rj = j < 0 ? R : runs + j;
             const int cj = j < 0 ? ck : (Rj->st->cur ^ 1);
             const unsigned nsj = Rj->B;
-            unsigned b0, b1;
-            segment_span(seg, nsk, nsj, b0, b1);
+            unsigned b0 = seg, b1 = seg;
+            if constexpr (ANY) segment_span(seg, nsk, nsj, b0, b1);
             for (unsigned sj = b0; sj <= b1; ++sj) {
                 const unsigned nj = j < 0 ? nk : min(Rj->vcount[cj][sj], Rj->Cv);
                 const K* jk = (const K*)Rj->vkeys[cj] + (size_t)sj * Rj->Cv;
@@ -1848,7 +1859,7 @@ __global__ void __launch_bounds__(128) k_gs_axpy(const RunDesc* __restrict__ run
                     bool is_new = false;
                     int q = -1;
                     // entries whose address lies in run k's segment
-                    if (i < nj && (nsj == nsk || segment_of(seg_hash(jk[i]), nsk) == seg)) {
+                    if (i < nj && (!ANY || nsj == nsk || segment_of(seg_hash(jk[i]), nsk) == seg)) {
                         q = table_insert(tk, T - 1u, jk[i], is_new);
                         if (q < 0) {
                             acc.full = true;

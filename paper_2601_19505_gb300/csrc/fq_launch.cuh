@@ -137,30 +137,41 @@ template <class K, int AMP, int KIND> struct Launch {
         k_ref_terms<K, KIND><<<(n + 63) / 64, 64, 0, s>>>(mp, (const K*)refs, y, n, off,
                                                           (K*)tkeys, th, tv, tseg, B);
     }
-    static void overlap(const RunDesc* d, const OverlapDesc* od, int grid, int wpb,
-                        unsigned table, cudaStream_t s) {
-        const size_t smem = (size_t)wpb * table * (sizeof(K) + sizeof(double) + sizeof(unsigned));
-        k_overlap<K, AMP, KIND><<<grid, wpb * 32, smem, s>>>(d, od);
-        k_overlap_row<<<1, kRowThreads, 0, s>>>(d, od, (unsigned)(grid * wpb));
+    template <bool ANY> static void overlap_v(const RunDesc* d, const OverlapDesc* od,
+                                              const JoinShape& j, cudaStream_t s) {
+        k_overlap<K, AMP, KIND, ANY><<<j.grid, j.wpb * 32, j.onchip() * overlap_slot(), s>>>(d, od);
+        k_overlap_row<<<1, kRowThreads, 0, s>>>(d, od, (unsigned)(j.grid * j.wpb));
+    }
+    static void overlap(const RunDesc* d, const OverlapDesc* od, const JoinShape& j, cudaStream_t s) {
+        if (j.any) overlap_v<true>(d, od, j, s);
+        else overlap_v<false>(d, od, j, s);
+    }
+    static constexpr size_t overlap_slot() { return sizeof(K) + sizeof(double) + sizeof(unsigned); }
+    template <class... P> static cudaError_t allow_smem(size_t smem, void (*kernel)(P...)) {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     }
     static cudaError_t prepare_overlap(size_t smem) {
-        return cudaFuncSetAttribute(k_overlap<K, AMP, KIND>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_smem(smem, k_overlap<K, AMP, KIND, false>);
+        return e == cudaSuccess ? allow_smem(smem, k_overlap<K, AMP, KIND, true>) : e;
     }
     static constexpr size_t gs_dots_slot() { return sizeof(K) + sizeof(double) + sizeof(unsigned); }
     static constexpr size_t gs_axpy_slot() { return sizeof(K) + sizeof(ACC) + sizeof(unsigned) + 1; }
-    static void gs(const RunDesc* d, const GsDesc* g, int k, int grid, int wpb, unsigned table,
-                   cudaStream_t s) {
-        k_gs_dots<K, AMP><<<grid, wpb * 32, (size_t)wpb * table * gs_dots_slot(), s>>>(d, g, k);
-        k_gs_alpha<<<1, kRowThreads, 0, s>>>(d, g, k, (unsigned)(grid * wpb));
-        k_gs_axpy<K, AMP, KIND><<<grid, wpb * 32, (size_t)wpb * table * gs_axpy_slot(), s>>>(d, g, k);
+    template <bool ANY> static void gs_v(const RunDesc* d, const GsDesc* g, int k, const JoinShape& j,
+                                         cudaStream_t s) {
+        const int t = j.wpb * 32;
+        k_gs_dots<K, AMP, ANY><<<j.grid, t, j.onchip() * gs_dots_slot(), s>>>(d, g, k);
+        k_gs_alpha<<<1, kRowThreads, 0, s>>>(d, g, k, (unsigned)(j.grid * j.wpb));
+        k_gs_axpy<K, AMP, KIND, ANY><<<j.grid, t, j.onchip() * gs_axpy_slot(), s>>>(d, g, k);
+    }
+    static void gs(const RunDesc* d, const GsDesc* g, int k, const JoinShape& j, cudaStream_t s) {
+        if (j.any) gs_v<true>(d, g, k, j, s);
+        else gs_v<false>(d, g, k, j, s);
     }
     static cudaError_t prepare_gs(size_t smem) {
-        cudaError_t e = cudaFuncSetAttribute(k_gs_dots<K, AMP>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_gs_axpy<K, AMP, KIND>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem(smem, k_gs_dots<K, AMP, false>);
+        if (e == cudaSuccess) e = allow_smem(smem, k_gs_dots<K, AMP, true>);
+        if (e == cudaSuccess) e = allow_smem(smem, k_gs_axpy<K, AMP, KIND, false>);
+        if (e == cudaSuccess) e = allow_smem(smem, k_gs_axpy<K, AMP, KIND, true>);
         return e;
     }
     static KernelSet make() {
@@ -192,7 +203,7 @@ template <class K, int AMP, int KIND> struct Launch {
         k.gs = gs;
         k.prepare_gs = prepare_gs;
         k.gs_slot_bytes = gs_dots_slot() > gs_axpy_slot() ? gs_dots_slot() : gs_axpy_slot();
-        k.overlap_slot_bytes = sizeof(K) + sizeof(double) + sizeof(unsigned);
+        k.overlap_slot_bytes = overlap_slot();
         return k;
     }
 };

@@ -36,14 +36,12 @@ struct KernelSet {
     void (*ref_terms)(const ModelParams&, const void* refs, const double* y, int n,
                       const unsigned* off, void* tkeys, double* th, double* tv, unsigned* tseg,
                       unsigned B, cudaStream_t);
-    // replica overlaps: `grid` blocks of `wpb` warps, then the row
-    void (*overlap)(const RunDesc* runs, const OverlapDesc* od, int grid, int wpb,
-                    unsigned table, cudaStream_t);
+    // replica overlaps, then the row
+    void (*overlap)(const RunDesc* runs, const OverlapDesc* od, const JoinShape&, cudaStream_t);
     size_t overlap_slot_bytes;  // one slot of an overlap table: key, FP64 amplitude, list entry
     cudaError_t (*prepare_overlap)(size_t smem);
-    // Gram-Schmidt of run k: dot products, coefficients, axpy (grid x wpb warps)
-    void (*gs)(const RunDesc* runs, const GsDesc* gs, int k, int grid, int wpb, unsigned table,
-               cudaStream_t);
+    // Gram-Schmidt of run k: dot products, coefficients, axpy
+    void (*gs)(const RunDesc* runs, const GsDesc* gs, int k, const JoinShape&, cudaStream_t);
     cudaError_t (*prepare_gs)(size_t smem);
     size_t gs_slot_bytes;  // one slot of the axpy table: key, value, list entry, flag
 };

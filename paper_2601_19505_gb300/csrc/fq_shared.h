@@ -150,6 +150,7 @@ struct OverlapDesc {
     int pa[FQ_MAX_PAIRS], pb[FQ_MAX_PAIRS];
     unsigned long long first[FQ_MAX_PAIRS + 1];  // pair p's first item: one per segment of A
     unsigned table;                // slots of a warp's table (power of 2)
+    unsigned char* tables;         // the warps' tables in device memory (null: on-chip)
     double* part;                  // per warp: P x (1 + nq) partial sums
     double* ring;                  // rows of width 1 + P (1 + nq)
     unsigned long long* head;      // rows written
@@ -163,8 +164,18 @@ struct OverlapDesc {
 struct GsDesc {
     int K;                  // spectral states
     unsigned table;         // slots of a warp's table (power of 2)
+    unsigned char* tables;  // the warps' tables in device memory (null: on-chip)
     double* part;           // per warp: 2 FQ_MAX_SPECTRAL partial dot products
     double* alpha;          // FQ_MAX_SPECTRAL coefficients of the run being orthogonalised
+};
+
+// launch of a join: persistent blocks of wpb warps with a table each
+struct JoinShape {
+    int grid, wpb;
+    unsigned table;  // slots (power of 2)
+    bool dev;        // the tables lie in device memory
+    bool any;        // they do, or the runs have unequal segment counts
+    size_t onchip() const { return dev ? 0 : (size_t)wpb * table; }  // slots of a block
 };
 
 struct LaunchCfg {
