@@ -1449,7 +1449,17 @@ static int batch_refresh(fq_batch* b) {
     if (!stale) return FQ_OK;
     CK(cudaStreamSynchronize(b->stream));
     batch_release(b);
-    return batch_build(b);
+    const int rc = batch_build(b);
+    if (rc) b->gens[0] = ~b->runs[0]->gen;  // incomplete: built again by the next call
+    return rc;
+}
+
+// the batch as it was before a setting that could not be built (should even
+// that fail, the next step tries again and reports it)
+static void batch_rebuild(fq_batch* b) {
+    b->gens[0] = ~b->runs[0]->gen;
+    const int rc = batch_refresh(b);
+    (void)rc;
 }
 
 static int batch_launch(fq_batch* b, int64_t n) {
@@ -2055,7 +2065,10 @@ extern "C" int fq_batch_set_overlaps(fq_batch* b, const int* g2_d, int n_g2) {
     // rebuild the descriptors and graphs with the overlap launch in each step
     batch_release(b);
     int rc = batch_build(b);
-    if (rc) overlaps_free(b);
+    if (rc) {
+        overlaps_free(b);
+        batch_rebuild(b);
+    }
     return rc;
 }
 
@@ -2082,9 +2095,7 @@ extern "C" int fq_batch_set_spectral(fq_batch* b, int K) {
     int rc = batch_build(b);
     if (rc) {
         gs_free(b);
-        batch_release(b);
-        const int rc2 = batch_build(b);
-        (void)rc2;
+        batch_rebuild(b);
     }
     return rc;
 }

@@ -68,6 +68,21 @@ def test_spectral_states_of_large_segments_match_oracle(model, entries):
     b.close()
 
 
+def test_larger_segments_are_refused_and_the_batch_steps_on():
+    h, m = pair(*CASES[0][0])
+    g, o = _runs(h, m, 45000, 2)
+    b = fq().Batch(g)
+    for call in (lambda: b.set_overlaps([]), lambda: b.set_spectral(2)):
+        with pytest.raises(fq().FqError):
+            call()
+    b.step(3)
+    b.sync()
+    for r, c in zip(g, o):
+        c.step(3)
+        assert_same_vector(r.export(), c.export(), rtol=1e-12)
+    b.close()
+
+
 def test_a_smaller_batch_leaves_an_earlier_one_its_tables():
     """Autotuning launches the join itself: it needs the on-chip memory that
     the batch was built for, whatever batches came after."""
