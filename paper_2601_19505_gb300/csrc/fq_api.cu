@@ -2127,7 +2127,10 @@ extern "C" int fq_batch_overlaps(fq_batch* b, double* rows, size_t cap, size_t* 
 
 extern "C" int fq_batch_autotune(fq_batch* b, int steps) {
     if (!b) return FQ_ERR_INVALID;
-    int rc = autotune(b, steps);
+    for (fq_run* r : b->runs)
+        if (r->no_spawn_buf) return FQ_ERR_NOMEM;
+    int rc = batch_refresh(b);  // a run may have grown: its old buffers are gone
+    if (!rc) rc = autotune(b, steps);
     if (rc) return rc;
     return fq_batch_sync(b);
 }
