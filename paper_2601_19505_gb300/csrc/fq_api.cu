@@ -1931,6 +1931,7 @@ static int autotune(fq_batch* b, int steps) {
 
 extern "C" int fq_run_autotune(fq_run* r, int steps) {
     if (!r || !r->seeded) return FQ_ERR_INVALID;
+    if (r->no_spawn_buf) return FQ_ERR_NOMEM;
     int rc = single_batch(r);
     if (!rc) rc = batch_refresh(r->single);
     if (rc) return rc;
@@ -1966,6 +1967,7 @@ extern "C" int fq_run_shape(fq_run* r, int* shape) {
 
 extern "C" int fq_run_profile(fq_run* r, int n, float* ms) {
     if (!r || !ms || n < 1 || n > 4096 || !r->seeded) return FQ_ERR_INVALID;
+    if (r->no_spawn_buf) return FQ_ERR_NOMEM;
     int rc = single_batch(r);
     if (!rc) rc = batch_refresh(r->single);
     if (rc) return rc;
