@@ -1245,27 +1245,39 @@ static std::vector<int> batch_arms(const fq_batch* b) {
     return {FQ_ANN_HASH_ARM, FQ_ANN_SORT_ARM};
 }
 
-// The shape a batch steps with unless the autotuner finds another.  With many
-// buckets for every warp, more warps of fewer registers: 64-bit addresses
-// spawn with 24 warps per SM (1e7 walkers on 20 sites 334 -> 298 us) and merge
-// with 20 (479 -> 432), 128-bit ones spawn with 20 in two waves of blocks
-// (1e8 walkers on 8 x 8 3277 -> 3111) but merge with 16, as does momentum
-// space (its diagonal wants the registers), which spawns with 24 warps in two
-// waves from one bucket a warp on (1e6 walkers on 32 modes 145 -> 137).  With
-// a few buckets a warp, the segments are cut for 16 warps per SM
-// (segments_for) and other shapes gained nothing.
+// The shape a batch steps with unless the autotuner finds another.  Segments
+// are cut for 16 warps per SM (segments_for), and with a few buckets a warp
+// that shape is the fastest.  With many, more warps of fewer registers (us a
+// step, spawn and merge, the 16-warp shape first):
+// - 64-bit addresses on a lattice, 24 warps spawning and 20 merging, from 16
+//   buckets a warp: 204 -> 184 and 292 -> 265 at 6e6 walkers on 20 sites, 334
+//   -> 298 and 479 -> 432 at 1e7; they cross between 4 (59.1 -> 58.4, 83.0 ->
+//   85.7) and 8 buckets (108 -> 102, 154 -> 147), integer walkers at 16 (230
+//   -> 231, 155 -> 153).
+// - 128-bit ones and momentum space, 20 warps spawning in two waves of blocks,
+//   from 20 buckets a warp: on 8 x 8 212 -> 215 at 6e6 walkers (16 buckets),
+//   264 -> 253 at 7.5e6, 3277 -> 3111 at 1e8 (FP32 204 -> 211, 253 -> 248; integer
+//   231 -> 236, 284 -> 279); in momentum space 748 -> 745 at 6e6 on 32 modes,
+//   889 -> 850 at 7.2e6, on 20 modes 826 -> 801.  Merging with more warps costs
+//   128-bit addresses 5 %.
+// - Momentum space below that, 24 warps in two waves, which three buckets for
+//   each of 16 warps fill evenly: with 3 a warp 144 -> 137 at 1e6 on 32 modes, 6
+//   290 -> 278, 12 554 -> 534; with other counts a wave stays part empty (1 a
+//   warp 54.6 -> 57.8, 2 94.0 -> 97.4, 4 192 -> 229, 5 242 -> 259).
 static LaunchCfg default_cfg(const fq_batch* b, unsigned slots, int ann) {
     const bool wide = b->ks->key_bytes == 16;
     const bool mom = b->runs[0]->ham.mp.kind == FQ_BH_MOM_1D;
     const unsigned warps = (unsigned)num_sms() * 16u;
     int sv = 0, waves = 1, mv = 0;
-    if (b->G >= 16u * warps) {
-        sv = wide && !mom ? 1 : 2;
-        waves = wide || mom ? 2 : 1;
-        mv = !wide && !mom && ann == FQ_ANN_HASH_ARM ? 1 : 0;
-    } else if (mom && b->G >= warps) {
+    if ((wide || mom) && b->G >= 20u * warps) {
+        sv = 1;
+        waves = 2;
+    } else if (mom && b->G % (3u * warps) == 0u) {
         sv = 2;
         waves = 2;
+    } else if (!wide && !mom && b->G >= 16u * warps) {
+        sv = 2;
+        mv = ann == FQ_ANN_HASH_ARM ? 1 : 0;
     }
     return make_cfg(b->ks, sv, waves, mv, slots, b->G, ann);
 }
