@@ -196,12 +196,10 @@ __device__ __forceinline__ unsigned pick(uint4 w, unsigned m) {
 }
 
 // segment hash; the segment is its high word scaled to the number of segments
-// (segment_of).  64-bit addresses: one
-// multiply by an odd constant (multiplicative hashing), unrelated to the
-// golden-ratio constant of the merge table's slot hash (with related
-// constants, small addresses that share a segment would also share a few
-// table slots).
-// 128-bit addresses fold the high word in by a multiply with another odd
+// (segment_of).  64-bit addresses: one multiply by an odd constant
+// (multiplicative hashing), unrelated to the golden-ratio constant of the merge
+// table's slot hash (with related constants, small addresses that share a
+// segment would also share a few table slots).  128-bit addresses fold the high word in by a multiply with another odd
 // constant, then take the same multiply: two 64-bit multiplies in all.
 __device__ __forceinline__ uint64_t seg_hash(uint64_t k) { return k * 0xD6E8FEB86659FD93ull; }
 __device__ __forceinline__ uint64_t seg_hash(u128 k) {

@@ -279,9 +279,8 @@ k_spawn(const RunDesc* __restrict__ runs, const unsigned* __restrict__ seg_run, 
     unsigned* const woff = (unsigned*)(wbase + SM::off_off);
     unsigned* const wm = (unsigned*)(wbase + SM::m_off);
     // the run's model parameters, copied into the warp's shared memory: read
-    // there, they are not reloaded
-    // through L1 after every spawn store (which the compiler cannot tell
-    // apart from the run descriptor)
+    // there, they are not reloaded through L1 after every spawn store (which
+    // the compiler cannot tell apart from the run descriptor)
     ModelParams* const wmp = (ModelParams*)(wbase + SM::mp_off);
     const ModelParams& mp = *wmp;
     unsigned g0, g1;
@@ -764,10 +763,8 @@ __device__ __forceinline__ bool is_taken(long long x) {
     return x == (long long)0x8000000000000000ull;
 }
 
-// Pi, compaction and the norm terms of one merged value, for a warp of lanes
-// (keep: the lane has a value)
-// compaction and the norm terms of the values a warp keeps (keep: the lane
-// stores `out` at `key`)
+// Compaction and the norm terms of the values a warp keeps (keep: the lane
+// stores `out` at `key`).
 template <class K, int AMP>
 __device__ __forceinline__ void merge_store(const StepConst& R, bool keep, K key,
                                             typename AmpT<AMP>::ACC out, K* __restrict__ ok,
@@ -803,6 +800,7 @@ __device__ __forceinline__ void merge_store(const StepConst& R, bool keep, K key
     nout += (unsigned)__popc(bal);
 }
 
+// Pi, then the above, for one merged value per lane (has: the lane has one).
 template <class K, int AMP>
 __device__ __forceinline__ void merge_emit(const StepConst& R, bool has, K key,
                                            typename AmpT<AMP>::ACC w, uint2 rkey, unsigned stepno,
@@ -1230,9 +1228,9 @@ k_merge(const RunDesc* __restrict__ runs, const unsigned* __restrict__ seg_run, 
     wait_for_previous();
     if (g0 >= g1) return;
     // The range's run: a range never crosses runs.  (A loop over the runs of a
-    // range, with totals flushed and restarted between them, counted wrongly
-    // for integer walkers: a batch's second run in a warp started from stale
-    // registers, while the same source steps right on a CPU.)
+    // range, with totals flushed and restarted between them, gave integer
+    // walkers of a batch's later runs wrong lengths and norms.  The cause was
+    // not found; the same source stepped right on a CPU.)
     const RunDesc* const R = runs + seg_run[g0];
     // lane 0 reads, the warp shares: another warp may set an error bit
     unsigned err = 0, cur = 0;
@@ -1723,7 +1721,8 @@ __global__ void __launch_bounds__(128) k_gs_dots(const RunDesc* __restrict__ run
         if (lane == 0 && seg + 1 < g1) {  // the next segment of every state into L2
             prefetch_segment<K, A>(Rk, ck, seg + 1);
             for (int j = 0; j < k; ++j)
-                if (!ANY || runs[j].B == nsk) prefetch_segment<K, A>(runs + j, runs[j].st->cur ^ 1, seg + 1);
+                if (!ANY || runs[j].B == nsk)
+                    prefetch_segment<K, A>(runs + j, runs[j].st->cur ^ 1, seg + 1);
         }
         const unsigned nk = min(Rk->vcount[ck][seg], Rk->Cv);
         const K* kk = (const K*)Rk->vkeys[ck] + (size_t)seg * Rk->Cv;
@@ -1837,7 +1836,8 @@ __global__ void __launch_bounds__(128) k_gs_axpy(const RunDesc* __restrict__ run
         if (lane == 0 && seg + 1 < g1) {  // the next segment of every state into L2
             prefetch_segment<K, A>(R, ck, seg + 1);
             for (int j = 0; j < k; ++j)
-                if (!ANY || runs[j].B == nsk) prefetch_segment<K, A>(runs + j, runs[j].st->cur ^ 1, seg + 1);
+                if (!ANY || runs[j].B == nsk)
+                    prefetch_segment<K, A>(runs + j, runs[j].st->cur ^ 1, seg + 1);
         }
         const unsigned nk = min(R->vcount[ck][seg], Cv);
         K* const kk = (K*)R->vkeys[ck] + (size_t)seg * Cv;

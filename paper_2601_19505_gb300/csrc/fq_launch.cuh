@@ -18,8 +18,8 @@ template <class K, int AMP, int KIND> struct Launch {
     template <int V> static void spawn_v(const LaunchCfg& c, const RunDesc* d, const unsigned* sr,
                                          unsigned G, cudaStream_t s) {
         constexpr int W = Var<V>::WPB;
-        launch_after(c.early_launch, k_spawn<K, AMP, KIND, V, 4>, c.spawn_grid, W * 32, spawn_smem(W), s, d, sr, G,
-                     c.spawn_cuts);
+        launch_after(c.early_launch, k_spawn<K, AMP, KIND, V, 4>, c.spawn_grid, W * 32,
+                     spawn_smem(W), s, d, sr, G, c.spawn_cuts);
     }
     static void spawn(const LaunchCfg& c, const RunDesc* d, const unsigned* sr, unsigned G,
                       cudaStream_t s) {
@@ -32,12 +32,14 @@ template <class K, int AMP, int KIND> struct Launch {
         constexpr int W = Var<V>::WPB;
         if (c.ann == FQ_ANN_SORT_ARM) {
             const size_t smem = (size_t)W * merge_warp_bytes<K, AMP, FQ_ANN_SORT_ARM>(c.slots);
-            launch_after(c.early_launch, k_merge<K, AMP, KIND, V, FQ_ANN_SORT_ARM>, c.merge_grid, W * 32, smem, s, d,
-                         sr, G, c.slots, c.sort_scratch, c.sort_elems, c.merge_cuts);
+            launch_after(c.early_launch, k_merge<K, AMP, KIND, V, FQ_ANN_SORT_ARM>, c.merge_grid,
+                         W * 32, smem, s, d, sr, G, c.slots, c.sort_scratch, c.sort_elems,
+                         c.merge_cuts);
         } else {
             const size_t smem = (size_t)W * merge_warp_bytes<K, AMP, FQ_ANN_HASH_ARM>(c.slots);
-            launch_after(c.early_launch, k_merge<K, AMP, KIND, V, FQ_ANN_HASH_ARM>, c.merge_grid, W * 32, smem, s, d,
-                         sr, G, c.slots, c.scratch, c.scratch_slots, c.merge_cuts);
+            launch_after(c.early_launch, k_merge<K, AMP, KIND, V, FQ_ANN_HASH_ARM>, c.merge_grid,
+                         W * 32, smem, s, d, sr, G, c.slots, c.scratch, c.scratch_slots,
+                         c.merge_cuts);
         }
     }
     static void merge(const LaunchCfg& c, const RunDesc* d, const unsigned* sr, unsigned G,
@@ -142,7 +144,8 @@ template <class K, int AMP, int KIND> struct Launch {
         k_overlap<K, AMP, KIND, ANY><<<j.grid, j.wpb * 32, j.onchip() * overlap_slot(), s>>>(d, od);
         k_overlap_row<<<1, kRowThreads, 0, s>>>(d, od, (unsigned)(j.grid * j.wpb));
     }
-    static void overlap(const RunDesc* d, const OverlapDesc* od, const JoinShape& j, cudaStream_t s) {
+    static void overlap(const RunDesc* d, const OverlapDesc* od, const JoinShape& j,
+                        cudaStream_t s) {
         if (j.any) overlap_v<true>(d, od, j, s);
         else overlap_v<false>(d, od, j, s);
     }
@@ -156,8 +159,8 @@ template <class K, int AMP, int KIND> struct Launch {
     }
     static constexpr size_t gs_dots_slot() { return sizeof(K) + sizeof(double) + sizeof(unsigned); }
     static constexpr size_t gs_axpy_slot() { return sizeof(K) + sizeof(ACC) + sizeof(unsigned) + 1; }
-    template <bool ANY> static void gs_v(const RunDesc* d, const GsDesc* g, int k, const JoinShape& j,
-                                         cudaStream_t s) {
+    template <bool ANY> static void gs_v(const RunDesc* d, const GsDesc* g, int k,
+                                         const JoinShape& j, cudaStream_t s) {
         const int t = j.wpb * 32;
         k_gs_dots<K, AMP, ANY><<<j.grid, t, j.onchip() * gs_dots_slot(), s>>>(d, g, k);
         k_gs_alpha<<<1, kRowThreads, 0, s>>>(d, g, k, (unsigned)(j.grid * j.wpb));

@@ -77,7 +77,8 @@ inline void launch_after(int early, void (*kernel)(P...), int grid, int block, s
     c.stream = s;
     c.attrs = at;
     c.numAttrs = 1;
-    cudaLaunchKernelEx(&c, kernel, P(args)...);
+    // as with <<<>>>, an error stays for cudaGetLastError or ends the capture
+    (void)cudaLaunchKernelEx(&c, kernel, P(args)...);
 }
 
 }  // namespace fq
