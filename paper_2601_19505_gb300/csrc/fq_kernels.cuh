@@ -958,6 +958,9 @@ __device__ __forceinline__ void merge_bucket(const RunDesc* R, unsigned seg, uns
             // (its sum is still 0; nearly every spawn reaches a new address).
             const unsigned grp = __match_any_sync(0xFFFFFFFFu, q);
             const unsigned bal = __ballot_sync(0xFFFFFFFFu, nw);
+            // the sums of the rounds before, before this round's reads of them
+            // (votes and matches order no memory)
+            __syncwarp();
             if (q >= 0) {
                 ACC sum = (ACC)v;
                 for (unsigned o = grp & (grp - 1u); o; o &= o - 1u)
@@ -966,9 +969,6 @@ __device__ __forceinline__ void merge_bucket(const RunDesc* R, unsigned seg, uns
             }
             if (nw) tl[nl + __popc(bal & ((1u << lane) - 1u))] = (unsigned)q;
             nl += __popc(bal);
-            // this round's sums before the next round's reads of them (the
-            // votes above order no memory)
-            __syncwarp();
         }
     }
     __syncwarp();
