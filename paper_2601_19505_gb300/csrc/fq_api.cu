@@ -92,6 +92,9 @@ struct fq_run {
     const KernelSet* ks;
     unsigned B, Cv, Cs, slots;  // slots: on-chip table slots per merge warp
     unsigned Cp;                // spawn slots per bucket in the dense primary region
+    unsigned group;             // segments that make a segment of the coarser map (1: none)
+    double cap_vec, cap_spawn;  // the capacities asked for
+    bool split_set;             // Cp was set by fq_run_set_spawn_split
     unsigned size_class;        // full buckets, rounded up to a power of two (joinable)
     SpawnRoom room;             // the buckets' spawn slots for a capacity
     double fill;                // steady-state spawns per bucket
@@ -676,7 +679,11 @@ extern "C" int fq_run_create(fq_run** out, const fq_ham* h, const fq_params* p, 
         l_ss = std::min(lcap, dim);
         s_ss = l_ss * (double)max_offdiag(h->mp);
     }
-    r->B = segments_for(s_ss, r->slots, num_sms());
+    const Segments sg = segments_for(s_ss, r->slots, num_sms());
+    r->B = sg.B;
+    r->group = sg.group;
+    r->cap_vec = lcap;
+    r->cap_spawn = scap;
     r->size_class = next_pow2((unsigned long long)full_segments(s_ss, r->slots));
     {
         // spawns arrive in clumps (one address receives spawns from many
@@ -1432,7 +1439,94 @@ static int batch_build(fq_batch* b) {
     return rc;
 }
 
+// One segment for every group of the run's segments: the vector into its other
+// buffer, the reference terms' offsets and the spawn buffers to match (smaller:
+// a full bucket's room was each small one's).
+static int run_regroup(fq_run* r) {
+    if (r->group < 2) return FQ_OK;
+    CK(cudaStreamSynchronize(r->stream));
+    const unsigned f = r->group, B = r->B / f;
+    int cur = 0;
+    std::vector<unsigned> cnt(r->B), off(r->B + 1);
+    CK(cudaMemcpy(&cur, &r->st->cur, sizeof cur, cudaMemcpyDeviceToHost));
+    CK(cudaMemcpy(cnt.data(), r->vcount[cur], sizeof(unsigned) * r->B, cudaMemcpyDeviceToHost));
+    CK(cudaMemcpy(off.data(), r->ref_off, sizeof(unsigned) * (r->B + 1), cudaMemcpyDeviceToHost));
+    unsigned most = 0;
+    std::vector<unsigned> noff(B + 1), bk;
+    for (unsigned g = 0; g < B; ++g) {
+        unsigned n = 0;
+        for (unsigned j = 0; j < f; ++j) n += std::min(cnt[g * f + j], r->Cv);
+        most = std::max(most, n);
+        noff[g] = off[g * f];
+        if (off[(g + 1) * f] > off[g * f]) bk.push_back(g);
+    }
+    noff[B] = off[r->B];
+    const unsigned Cv = std::min(f * r->Cv, std::max(vec_slots(r->cap_vec, B), (most + 31u) / 32u * 32u));
+    SpawnRoom room = r->room;
+    room.B = B;
+    room.rooms = std::min(room.rooms, (double)B);
+    const unsigned Cs = std::min(f * r->Cs, room.slots(r->cap_spawn));
+    // the old spawn buffers are large enough should the new ones not fit
+    void* nk = dev_alloc(r, r->ks->spawn_key_stride * (size_t)B * Cs);
+    void* nv = dev_alloc(r, std::max<size_t>(16, r->ks->spawn_val_stride * (size_t)B * Cs));
+    if (nk && nv) std::swap(nk, r->skeys), std::swap(nv, r->samps);
+    if (nk) dev_free(r, nk);
+    if (nv) dev_free(r, nv);
+    r->ks->regroup(r->vkeys[cur], r->vamps[cur], r->Cv, r->vcount[cur], f, B, r->vkeys[cur ^ 1],
+                   r->vamps[cur ^ 1], Cv, r->vcount[cur ^ 1], r->stream);
+    CK(cudaGetLastError());
+    cur ^= 1;
+    CK(cudaMemcpyAsync(&r->st->cur, &cur, sizeof cur, cudaMemcpyHostToDevice, r->stream));
+    CK(cudaMemcpyAsync(r->ref_off, noff.data(), sizeof(unsigned) * (B + 1), cudaMemcpyHostToDevice,
+                       r->stream));
+    CK(cudaMemcpyAsync(r->ref_bkt, bk.data(), sizeof(unsigned) * bk.size(), cudaMemcpyHostToDevice,
+                       r->stream));
+    const double s_ss = r->fill * r->B;
+    r->n_ref_bkt = (unsigned)bk.size();
+    r->B = B;
+    r->group = 1;
+    r->fill *= f;
+    r->Cv = Cv;
+    r->Cs = Cs;
+    r->room = room;
+    r->Cp = r->split_set ? std::min(r->Cp * f, Cs) : primary_slots(s_ss, B, room.k, Cs);
+    table_sizes(r);
+    r->has_tuned = false;  // a tuned shape was timed with the small buckets
+    r->gen++;
+    CK(sync_self(r));
+    return FQ_OK;
+}
+
+// The small buckets of small runs spread one run over the warps.  A batch that
+// fills the warps without them pays their fixed costs (share_cuts) for nothing:
+// its runs' segments are grouped where that makes the largest share of a warp
+// smaller.  Runs of 1e4 walkers on 12 sites, us a step with small buckets and
+// grouped: 16 runs 42.8 and 47.8, 24 runs 52.4 and 49.4, 64 runs 105 and 80, 1024
+// runs 1632 and 1048 (the rule's line lies at 21 runs); of 1e5 on 20 sites: 2
+// runs 37.2 and 59.0, 6 runs 89.4 and 87.4, 64 runs 661 and 484 (at 3 runs; 57.0
+// and 62.2 there).
+static int batch_groups(fq_run* const* runs, int n) {
+    double fine = 0.0, grouped = 0.0, most_fine = 0.0, most_grouped = 0.0;
+    for (int i = 0; i < n; ++i) {
+        const fq_run* r = runs[i];
+        const double a = 32.0 + r->fill, b = 32.0 + r->fill * r->group;
+        fine += r->B * a;
+        grouped += r->B / r->group * b;
+        most_fine = std::max(most_fine, a);
+        most_grouped = std::max(most_grouped, b);
+    }
+    const double warps = num_sms() * 16.0;
+    if (std::max(grouped / warps, most_grouped) >= std::max(fine / warps, most_fine)) return FQ_OK;
+    int rc = FQ_OK;
+    for (int i = 0; i < n && !rc; ++i) rc = run_regroup(runs[i]);
+    return rc;
+}
+
 static int batch_new(fq_run* const* runs, int n, bool owned, fq_batch** out) {
+    if (n > 1) {
+        const int rc = batch_groups(runs, n);
+        if (rc) return rc;
+    }
     fq_batch* b = new (std::nothrow) fq_batch();
     if (!b) return FQ_ERR_NOMEM;
     b->runs.assign(runs, runs + n);
@@ -1631,6 +1725,8 @@ extern "C" int fq_run_reserve(fq_run* r, size_t capacity_vec, size_t capacity_sp
     if (rc) return rc;
     const unsigned Cv = std::max(vec_slots((double)capacity_vec, r->B), r->Cv);
     const unsigned Cs = std::max(r->room.slots((double)capacity_spawn), r->Cs);
+    r->cap_vec = std::max(r->cap_vec, (double)capacity_vec);
+    r->cap_spawn = std::max(r->cap_spawn, (double)capacity_spawn);
     if (Cv == r->Cv && Cs == r->Cs) return FQ_OK;
     const size_t kb = r->ks->key_bytes, ab = r->ks->amp_bytes, sb = r->ks->spawn_bytes;
     int cur = 0;
@@ -1718,6 +1814,7 @@ extern "C" int fq_run_set_spawn_split(fq_run* r, unsigned primary) {
     if (rc) return rc;
     if (primary % 32u || primary > r->Cs) return FQ_ERR_INVALID;
     r->Cp = primary;
+    r->split_set = true;
     r->gen++;
     CK(sync_self(r));
     return FQ_OK;

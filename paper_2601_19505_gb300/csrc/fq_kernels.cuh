@@ -1961,6 +1961,29 @@ __global__ void k_restride(const K* __restrict__ ok, const A* __restrict__ oa, u
     }
 }
 
+// the segments of each group, of stride `oc`, become one segment of stride
+// `nc` (one warp per group)
+template <class K, class A>
+__global__ void k_regroup(const K* __restrict__ ok, const A* __restrict__ oa, unsigned oc,
+                          const unsigned* __restrict__ cnt, unsigned group, unsigned groups,
+                          K* __restrict__ nk, A* __restrict__ na, unsigned nc,
+                          unsigned* __restrict__ ncnt) {
+    const unsigned g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31u;
+    if (g >= groups) return;
+    unsigned n = 0;
+    for (unsigned j = 0; j < group; ++j) {
+        const size_t from = (size_t)(g * group + j);
+        const unsigned c = min(cnt[from], oc);
+        for (unsigned i = lane; i < c; i += 32)
+            if (n + i < nc) {
+                nk[(size_t)g * nc + n + i] = ok[from * oc + i];
+                na[(size_t)g * nc + n + i] = oa[from * oc + i];
+            }
+        n += c;
+    }
+    if (lane == 0) ncnt[g] = min(n, nc);
+}
+
 // amplitude of each query address in the vector (0 when absent): the
 // address's segment is scanned
 template <class K, int AMP>

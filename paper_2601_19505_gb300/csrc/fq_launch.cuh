@@ -110,6 +110,12 @@ template <class K, int AMP, int KIND> struct Launch {
         k_gather<K, A><<<B < 4096 ? B : 4096, 256, 0, s>>>((const K*)keys, (const A*)amps, cap, cnt,
                                                            off, B, (K*)okeys, ovals, segs);
     }
+    static void regroup(const void* ok, const void* oa, unsigned oc, const unsigned* cnt,
+                        unsigned group, unsigned groups, void* nk, void* na, unsigned nc,
+                        unsigned* ncnt, cudaStream_t s) {
+        k_regroup<K, A><<<(groups + 3) / 4, 128, 0, s>>>((const K*)ok, (const A*)oa, oc, cnt, group,
+                                                         groups, (K*)nk, (A*)na, nc, ncnt);
+    }
     static void restride(const void* ok, const void* oa, unsigned oc, const unsigned* cnt,
                          unsigned B, void* nk, void* na, unsigned nc, cudaStream_t s) {
         k_restride<K, A><<<B < 8192 ? B : 8192, 128, 0, s>>>((const K*)ok, (const A*)oa, oc, cnt, B,
@@ -198,6 +204,7 @@ template <class K, int AMP, int KIND> struct Launch {
         k.gather_spawns = gather_spawns;
         k.lookup = lookup;
         k.restride = restride;
+        k.regroup = regroup;
         k.column = column;
         k.ref_count = ref_count;
         k.ref_terms = ref_terms;

@@ -25,6 +25,8 @@ struct KernelSet {
                        const unsigned* off, unsigned B, void* okeys, double* ovals,
                        const unsigned* segs, cudaStream_t);
     void (*lookup)(const RunDesc* d, const void* keys, size_t n, double* out, cudaStream_t);
+    void (*regroup)(const void* ok, const void* oa, unsigned oc, const unsigned* cnt, unsigned group,
+                    unsigned groups, void* nk, void* na, unsigned nc, unsigned* ncnt, cudaStream_t);
     void (*restride)(const void* ok, const void* oa, unsigned oc, const unsigned* cnt, unsigned B,
                      void* nk, void* na, unsigned nc, cudaStream_t);
     void (*gather_spawns)(const void* keys, const void* vals, unsigned cap, unsigned Cp,

@@ -17,6 +17,12 @@ inline double full_segments(double s_ss, unsigned slots) {
     return std::max(1.0, std::ceil(std::min(s_ss / (slots / 3.0), 268000000.0)));
 }
 
+// Segments of a run: B of them, in groups of `group` that are one segment of a
+// coarser map (segment_of scales the hash, so consecutive segments are).
+struct Segments {
+    unsigned B, group;
+};
+
 // Segments for s_ss spawns a step.  Large runs: full buckets, and a multiple
 // of the warps that are resident at once (16 per SM in the default launch
 // shape), so that every warp takes the same number: with a power of two, 1e6
@@ -25,13 +31,18 @@ inline double full_segments(double s_ss, unsigned slots) {
 // instead of 646912 of 170 (2 %).  Below one full bucket per warp, smaller
 // buckets on more warps, down to one round of 32 spawns: a step of 1e4
 // walkers on 12 sites took 39 us with buckets of 86 spawns and takes 33 with
-// 32, 1e5 on 20 sites 42 and 37.  Less than 64 such buckets (2000 walkers, in
-// spaces where a few addresses draw most of the spawns) stay at 100.
-inline unsigned segments_for(double s_ss, unsigned slots, int sms) {
+// 32, 1e5 on 20 sites 42 and 37.  They come in groups that make about a full
+// bucket, for batches that fill the warps without them (batch_groups in
+// fq_api.cu).  Less than 64 such buckets (2000 walkers, in spaces where a few
+// addresses draw most of the spawns) stay at 100.
+inline Segments segments_for(double s_ss, unsigned slots, int sms) {
     const double warps = sms * 16.0, full = full_segments(s_ss, slots);
-    if (full > warps) return (unsigned)(std::ceil(full / warps) * warps);
-    const double fine = std::ceil(s_ss / (s_ss < 64.0 * 32.0 ? 100.0 : 32.0));
-    return (unsigned)std::max(1.0, std::min(warps, fine));
+    if (full > warps) return {(unsigned)(std::ceil(full / warps) * warps), 1};
+    if (s_ss < 64.0 * 32.0) return {(unsigned)std::max(1.0, std::ceil(s_ss / 100.0)), 1};
+    const double fine = std::min(warps, std::ceil(s_ss / 32.0));
+    const double group = std::max(1.0, std::floor(fine / full + 0.5));
+    const double groups = std::min(std::ceil(fine / group), std::floor(warps / group));
+    return {(unsigned)(groups * group), (unsigned)group};
 }
 
 // entries per segment for `total` over B segments

@@ -9,7 +9,7 @@ from gpu_helpers import assert_same_vector, fq, pair
 
 pytestmark = pytest.mark.gpu
 
-# 344 segments; entries per segment, so that an overlap table is beyond 200 KB
+# 345 segments; entries per segment, so that an overlap table is beyond 200 KB
 # (16384 slots of 20 bytes, 8192 of 28) and a two-state one below 800 KB
 CASES = [((O.REAL_1D, 20, 1, 20, 1.0, 2.0), 9300), ((O.REAL_1D, 33, 1, 33, 1.0, 20.0), 4000)]
 

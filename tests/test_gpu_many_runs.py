@@ -25,7 +25,10 @@ def test_many_equal_runs_step_alike():
     b.step(6)
     b.sync()
     for r in together:
-        assert r.history(cap=16).tobytes() == rows.tobytes()
+        h6 = r.history(cap=16)
+        for f in rows.dtype.names:  # the energy's terms are added segment by segment
+            assert (np.allclose(h6[f], rows[f], rtol=1e-14, atol=0) if f == "hproj"
+                    else np.array_equal(h6[f], rows[f])), f
     for r in (together[0], together[950], together[-1]):
         k, a = r.export()
         assert np.array_equal(k, ka) and np.array_equal(a, aa)

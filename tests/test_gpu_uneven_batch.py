@@ -40,10 +40,11 @@ def test_uneven_batch_rows_are_those_of_the_runs_alone(shape, mode, arm):
         for f in ("step", "len", "exact_steps", "inexact_steps", "n_spawns"):
             assert np.array_equal(x[f], y[f]), (i, f)
         for f in ("norm", "shift", "hproj", "vproj"):
-            if mode == 0:
+            if mode == 0 and f != "hproj":
                 assert np.array_equal(x[f], y[f]), (i, f)
-            else:
-                assert np.allclose(x[f], y[f], rtol=tol, atol=tol * np.max(np.abs(y[f]))), (i, f)
+            else:  # the energy's terms are added segment by segment
+                rtol = max(tol, 1e-14)
+                assert np.allclose(x[f], y[f], rtol=rtol, atol=rtol * np.max(np.abs(y[f]))), (i, f)
         assert_same_vector(r.export(), a.export(), rtol=tol, what="run %d" % i)
         a.close()
     b.close()

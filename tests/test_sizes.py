@@ -12,7 +12,8 @@ CSRC = os.path.join(ROOT, "paper_2601_19505_gb300", "csrc")
 WRAP = """
 #include "fq_sizes.h"
 using namespace fq;
-extern "C" unsigned segs(double s, unsigned slots, int sms) { return segments_for(s, slots, sms); }
+extern "C" unsigned segs(double s, unsigned slots, int sms) { return segments_for(s, slots, sms).B; }
+extern "C" unsigned group(double s, unsigned slots, int sms) { return segments_for(s, slots, sms).group; }
 extern "C" double full(double s, unsigned slots) { return full_segments(s, slots); }
 extern "C" unsigned vec(double t, unsigned B) { return vec_slots(t, B); }
 extern "C" unsigned spawn(unsigned B, double full, double usual, double t) {
@@ -33,7 +34,8 @@ def lib(tmp_path_factory):
     L = ctypes.CDLL(str(d / "libsizes.so"))
     D, U = ctypes.c_double, ctypes.c_uint
     L.full.restype = L.total.restype = D
-    L.segs.restype = L.vec.restype = L.spawn.restype = U
+    L.segs.restype = L.group.restype = L.vec.restype = L.spawn.restype = U
+    L.group.argtypes = [D, U, ctypes.c_int]
     L.segs.argtypes, L.full.argtypes, L.vec.argtypes = [D, U, ctypes.c_int], [D, U], [D, U]
     L.spawn.argtypes, L.total.argtypes = [U, D, D, D], [U, D, D, U]
     return L
@@ -65,3 +67,21 @@ def test_capacities(lib, target, slots):
         t *= 2.0
     for t in (1e3, target, 1e8):
         assert lib.vec(t, B) * B >= t
+
+
+@pytest.mark.parametrize("slots", [256, 512])
+@pytest.mark.parametrize("sms", [1, 132, 152])
+def test_groups_of_small_buckets_are_about_full_ones(lib, slots, sms):
+    t = 10.0
+    while t < 1e8:
+        B, group, full = lib.segs(t, slots, sms), lib.group(t, slots, sms), lib.full(t, slots)
+        warps = 16 * sms
+        assert B % group == 0
+        if full > warps or t < 2048.0:
+            assert group == 1
+        else:
+            # no more buckets than warps; a group fills 1 to 3 sixths of a table
+            assert B <= warps
+            if group > 1:
+                assert slots / 6.0 <= t * group / B <= slots / 2.0
+        t *= 1.03
