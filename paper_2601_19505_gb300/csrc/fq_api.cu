@@ -1305,12 +1305,17 @@ static std::vector<LaunchCfg> batch_shapes(fq_batch* b, unsigned slots) {
     return v;
 }
 
+static std::vector<ShareRun> share_runs(const fq_batch* b) {
+    std::vector<ShareRun> v;
+    for (const fq_run* r : b->runs) v.push_back({r->B, r->fill});
+    return v;
+}
+
 // every launch shape's shares of the batch's segments (none for a single run:
 // equal counts)
 static int batch_cuts(fq_batch* b) {
     if (b->runs.size() < 2) return FQ_OK;
-    std::vector<ShareRun> runs;
-    for (const fq_run* r : b->runs) runs.push_back({r->B, r->fill});
+    const std::vector<ShareRun> runs = share_runs(b);
     std::vector<unsigned> all, cuts;
     std::vector<std::pair<unsigned, size_t>> have;  // warps, offset of their cuts
     bool ok = true;
@@ -1362,6 +1367,12 @@ static int batch_build(fq_batch* b) {
     CK(cudaMemcpy(b->d_seg_run, seg_run.data(), sizeof(unsigned) * base, cudaMemcpyHostToDevice));
     CK(b->ks->prepare(200u * 1024u));
     b->shapes = batch_shapes(b, slots);
+    if (nr > 1) {  // the default shape, of one wave or two, in as many as its shares need
+        LaunchCfg& c = b->shapes[0];
+        const std::vector<ShareRun> runs = share_runs(b);
+        c.spawn_grid *= (int)share_waves(runs, (unsigned)(c.spawn_grid * c.spawn_wpb));
+        c.merge_grid *= (int)share_waves(runs, (unsigned)(c.merge_grid * c.merge_wpb));
+    }
     for (LaunchCfg& c : b->shapes) {  // every run has a warp of its own
         c.spawn_grid = std::max(c.spawn_grid, ((int)nr + c.spawn_wpb - 1) / c.spawn_wpb);
         c.merge_grid = std::max(c.merge_grid, ((int)nr + c.merge_wpb - 1) / c.merge_wpb);

@@ -41,8 +41,7 @@ inline Segments segments_for(double s_ss, unsigned slots, int sms) {
     if (s_ss < 64.0 * 32.0) return {(unsigned)std::max(1.0, std::ceil(s_ss / 100.0)), 1};
     const double fine = std::min(warps, std::ceil(s_ss / 32.0));
     const double group = std::max(1.0, std::floor(fine / full + 0.5));
-    const double groups = std::min(std::ceil(fine / group), std::floor(warps / group));
-    return {(unsigned)(groups * group), (unsigned)group};
+    return {(unsigned)(std::floor(fine / group) * group), (unsigned)group};
 }
 
 // entries per segment for `total` over B segments
