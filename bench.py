@@ -59,7 +59,8 @@ ANN_CODE = {"auto": 0, "sort": 1, "hash": 2}
 STATS_D2H_BYTES = 4 + 192  # the error word, then the 192-byte run state
 # the sources a committed ncu summary depends on: the kernels, and the host
 # code that sizes the buffers, tables and launch shapes they run with
-KERNEL_FILES = ["fq_kernels.cuh", "fq_device.cuh", "fq_shared.h", "fq_launch.cuh", "fq_api.cu"]
+KERNEL_FILES = ["fq_kernels.cuh", "fq_device.cuh", "fq_shared.h", "fq_launch.cuh", "fq_api.cu",
+                "fq_sizes.h", "fq_shares.h"]
 
 
 def describe(cfg, name):
