@@ -1512,10 +1512,10 @@ static int run_regroup(fq_run* r) {
 // fills the warps without them pays their fixed costs (share_cuts) for nothing:
 // its runs' segments are grouped where that makes the largest share of a warp
 // smaller.  Runs of 1e4 walkers on 12 sites, us a step with small buckets and
-// grouped: 16 runs 42.8 and 47.8, 24 runs 52.4 and 49.4, 64 runs 105 and 80, 1024
-// runs 1632 and 1048 (the rule's line lies at 21 runs); of 1e5 on 20 sites: 2
-// runs 37.2 and 59.0, 6 runs 89.4 and 87.4, 64 runs 661 and 484 (at 3 runs; 57.0
-// and 62.2 there).
+// grouped: 4 runs 24.3 and 37.2, 16 runs 42.4 and 42.0, 24 runs 52.6 and 43.0, 64
+// runs 105 and 88, 1024 runs 1263 and 833 (the rule's line lies at 18 runs); of
+// 1e5 on 20 sites: 2 runs 37.0 and 54.4, 3 runs 56.9 and 55.2, 16 runs 176 and
+// 149, 64 runs 657 and 484 (at 3 runs).
 static int batch_groups(fq_run* const* runs, int n) {
     double fine = 0.0, grouped = 0.0, most_fine = 0.0, most_grouped = 0.0;
     for (int i = 0; i < n; ++i) {

@@ -39,9 +39,9 @@ inline double share_bound(const std::vector<ShareRun>& runs, unsigned nw) {
 
 // Waves of `resident` warps that a batch's shares are cut for.  One, unless the
 // shares of so few warps, each within a run, leave many without work: 1024 runs
-// of 68 segments are two shares each on 2432 warps (84 % of them busy), 1900
-// one (78 %).  In three and four waves of smaller shares they are 97 and 96 %
-// (1024 runs of 1e4 walkers 1046 -> 851 us a step, 1900 2239 -> 1505).  A share
+// of 86 segments are two shares each on 2432 warps (84 % of them busy), 1900
+// one (78 %).  In three and four waves of smaller shares they are 93 and 93 %
+// (1024 runs of 1e4 walkers 1046 -> 834 us a step, 1900 2239 -> 1499).  A share
 // of its own costs its warp a start, taken as 100 spawns: three replicas with
 // shares of four segments were 3 % slower in three waves of shares of one.
 inline unsigned share_waves(const std::vector<ShareRun>& runs, unsigned resident) {

@@ -33,15 +33,21 @@ struct Segments {
 // walkers on 12 sites took 39 us with buckets of 86 spawns and takes 33 with
 // 32, 1e5 on 20 sites 42 and 37.  They come in groups that make about a full
 // bucket, for batches that fill the warps without them (batch_groups in
-// fq_api.cu).  Less than 64 such buckets (2000 walkers, in spaces where a few
+// fq_api.cu), of one segment more or fewer where that takes in more of them (1e4
+// walkers 344 in fours instead of 340 in fives: 1 % of the step).  Less than 64 such buckets (2000 walkers, in spaces where a few
 // addresses draw most of the spawns) stay at 100.
 inline Segments segments_for(double s_ss, unsigned slots, int sms) {
     const double warps = sms * 16.0, full = full_segments(s_ss, slots);
     if (full > warps) return {(unsigned)(std::ceil(full / warps) * warps), 1};
     if (s_ss < 64.0 * 32.0) return {(unsigned)std::max(1.0, std::ceil(s_ss / 100.0)), 1};
     const double fine = std::min(warps, std::ceil(s_ss / 32.0));
-    const double group = std::max(1.0, std::floor(fine / full + 0.5));
-    return {(unsigned)(std::floor(fine / group) * group), (unsigned)group};
+    const double near = std::max(1.0, std::floor(fine / full + 0.5));
+    auto whole = [&](double g) { return std::floor(fine / g) * g; };  // in whole groups
+    double group = near;
+    if (whole(near) < 0.99 * fine)
+        for (double g : {near - 1.0, near + 1.0})
+            if (g > 1.0 && whole(g) > whole(group)) group = g;
+    return {(unsigned)whole(group), (unsigned)group};
 }
 
 // entries per segment for `total` over B segments

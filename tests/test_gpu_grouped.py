@@ -31,7 +31,7 @@ def test_grouped_runs_follow_the_oracle(model, mode):
     before = [a.capacity() for a in g]
     b = fq().Batch(g)
     after = [a.capacity() for a in g]
-    assert all(x != y for x, y in zip(before, after))  # 340 segments are 68 now
+    assert all(x != y for x, y in zip(before, after))  # 344 segments are 86 now
     b.step(5)
     b.sync()
     for i, c in o:

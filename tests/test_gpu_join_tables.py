@@ -9,7 +9,7 @@ from gpu_helpers import assert_same_vector, fq, pair
 
 pytestmark = pytest.mark.gpu
 
-# 340 segments; entries per segment, so that an overlap table is beyond 200 KB
+# 344 segments; entries per segment, so that an overlap table is beyond 200 KB
 # (16384 slots of 20 bytes, 8192 of 28) and a two-state one below 800 KB
 CASES = [((O.REAL_1D, 20, 1, 20, 1.0, 2.0), 9300), ((O.REAL_1D, 33, 1, 33, 1.0, 20.0), 4000)]
 
@@ -21,7 +21,7 @@ def _runs(h, m, entries, n):
     for i in range(n):
         p = dict(mode=1, dt=1e-3, target=1e4, seed=9, run_id=i)
         amps = rng.integers(8, 80, len(keys)) * rng.choice([-0.125, 0.125], len(keys))
-        r = fq().Run(h, fq().default_params(capacity_vec=340 * entries, **p))
+        r = fq().Run(h, fq().default_params(capacity_vec=344 * entries, **p))
         c = O.Run(m, O.default_params(**p))
         r.seed(fq().keys_from_ints(keys), amps, m.diagonal(m.start()), 0)
         c.seed(keys, amps, m.diagonal(m.start()), 0)

@@ -10,7 +10,7 @@ from gpu_helpers import assert_same_vector, fq, pair
 
 pytestmark = pytest.mark.gpu
 
-TARGETS = [1.3e4, 1.9e4, 1e4]  # 445, 650 and 340 segments
+TARGETS = [1.3e4, 1.9e4, 1e4]  # 445, 650 and 344 segments
 
 
 def _runs(h, m, targets, mode, dt, starts):
@@ -101,7 +101,7 @@ def test_runs_of_another_size_class_are_refused():
 @pytest.mark.parametrize("mode,rtol", [(1, 1e-12), (0, 1e-12), (2, 1e-5)],
                          ids=["REAL64", "INT", "REAL32"])
 def test_warps_that_cross_pairs_match_oracle(mode, rtol):
-    """Eight replicas of 340 segments: 9520 items of 28 pairs, more than the
+    """Eight replicas of 344 segments: 9632 items of 28 pairs, more than the
     join's warps, so that some begin one pair's sums after another's."""
     h, m = pair(O.REAL_1D, 12, 1, 12, 1.0, 4.0)
     g, o = _runs(h, m, [1e4] * 8, mode, 1e-3, [([m.start()], [1000.0])] * 8)

@@ -9,7 +9,7 @@ pytestmark = pytest.mark.gpu
 
 
 def test_many_equal_runs_step_alike():
-    # 1900 runs of 34 segments (170 in groups of 5): more runs than half the warps of either kernel
+    # 1900 runs of 43 segments (172 in groups of 4): more runs than half the warps of either kernel
     h = fq().Hamiltonian(1, 8, 1, 8, 1.0, 3.0)
 
     def make():

@@ -9,7 +9,7 @@ pytestmark = pytest.mark.gpu
 
 
 def test_reserving_twice_the_capacity_grows_the_buckets():
-    # 12 sites, 340 buckets, integer walkers at the start address: every attempt
+    # 12 sites, 344 buckets, integer walkers at the start address: every attempt
     # of the 4000 is a spawn (dt 24 sqrt(2) = 1.02) to one of 24 neighbours, all
     # in different buckets, 167 each on average (deviation 13).  3000 spawns a
     # step are 160 slots per bucket, 6000 are 224.
