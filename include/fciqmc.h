@@ -315,7 +315,11 @@ int fq_run_profile(fq_run *r, int n, float *ms);
 
 /* A batch: B runs (same Hamiltonian kind, address width, mode and
  * annihilation strategy; any sizes and other parameters) stepped together by
- * one launch per kernel per step. */
+ * one launch per kernel per step.  In a batch that fills the GPU, runs below
+ * about 2.5e5 walkers change to fewer, fuller segments: their capacities
+ * (fq_run_capacity), spawn buffers and default launch shape change, their
+ * trajectories do not (sums over segments round differently).  Synchronises;
+ * device memory comes from the runs' allocators. */
 int fq_batch_create(fq_batch **out, fq_run *const *runs, int B);
 void fq_batch_destroy(fq_batch *b);
 int fq_batch_step(fq_batch *b, int64_t n);

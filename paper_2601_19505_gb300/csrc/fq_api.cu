@@ -1086,8 +1086,8 @@ constexpr size_t kJoinSmem = 200u * 1024u;
 // tables of up to four warps a block, and as many blocks as the SM's 228 KB
 // hold (1 KB of it reserved per block), at most 8 an SM.  A table beyond 200 KB
 // lies in device memory, four warps an SM (`tables`, allocated anew; up to
-// 800 KB each): segments of a capacity some times the derived one, which
-// segment counts that are powers of two kept below 200 KB or not.
+// 800 KB each): segments of a capacity several times the derived one, up to
+// twice as large as with the next power of two of segments.
 static int join_shape(size_t slot, unsigned T, unsigned long long items, JoinShape& j,
                       unsigned char*& tables) {
     const size_t one = (size_t)T * slot;
